@@ -260,16 +260,19 @@ fdtd_status fdtd_set_filter_width(fdtd_ctx *ctx, double sigma);
  * default.  Such passes are not replayed as CUDA graphs.
  *
  * 2D E_z contexts: with steps > 1 the forward (and recompute) and the
- * full-history adjoint advance up to min(steps, 8) steps per launch (4 in
- * FP64) by temporal blocking: a block owns a square tile (16 to 32 nodes a
- * side, the smallest whose tiles fit one wave of blocks), loads it with a
- * halo of that many nodes into shared memory, advances all the steps there
- * and writes back its tile, so no block waits for another.  Small grids,
- * whose launch-per-step kernels are single partial waves, gain: the default
- * is 8 for FP32 grids of at most one 32 x 32 tile per SM (316^2: 7.1 -> 2.9
- * us per forward step) and 1 otherwise (a 640^2 grid or an FP64 one runs
- * slower blocked).  Results agree with the launch-per-step path to rounding
- * (the per-node arithmetic of its generic path).
+ * adjoint advance up to min(steps, 8) steps per launch (4 in FP64, and 4 to 8
+ * in FP32 as suits the grid) by temporal blocking: a block holds a tile of
+ * the grid and a halo of that many nodes in registers, advances all the
+ * steps there and writes back its tile, so no block waits for another.  Left
+ * unset, grids of at most 2^21 nodes (FP64: 2^20) run so and larger ones with
+ * one launch per step (316^2 FP32: 6.9 us per forward step with one launch
+ * per step, 1.0 blocked; 160^2 FP64: 12.1 and 3.3).  Results of a run left
+ * unset are those of one launch per step bit for bit in the fields, W~ and
+ * the gap history (for a Courant number that is a power of two; to rounding
+ * otherwise), except on FP32 grids of at most one 32 x 32 tile per SM
+ * and with steps > 1, where a Drude node's two products are rounded in the
+ * other order; the gradient's FP32 sums of one launch are kept as exact
+ * pairs before they go into the FP64 accumulator (1e-14 relative).
  *
  * 3D contexts ignore the setting (see fdtd_set_wavefront). */
 fdtd_status fdtd_set_steps_per_launch(fdtd_ctx *ctx, int steps);
@@ -441,7 +444,9 @@ fdtd_status fdtd_set_graphs(fdtd_ctx *ctx, int mode);
  * that part of the state stays in L2 from one step to the next.  0 turns
  * the windows off, gives the set-aside back and demotes the lines marked
  * persisting; fdtd_destroy does the same for a context that has it on.
- * Results are unchanged.  FDTD_EINVAL outside [0, 1].  Default: off. */
+ * Results are unchanged.  While a context runs temporally blocked launches
+ * (fdtd_set_steps_per_launch), which take no window, nothing is set aside.
+ * FDTD_EINVAL outside [0, 1].  Default: off. */
 fdtd_status fdtd_set_l2_residency(fdtd_ctx *ctx, double fraction);
 
 /* Wait for the context's stream and report (then clear) device-side errors:

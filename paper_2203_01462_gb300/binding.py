@@ -299,8 +299,8 @@ class Solver:
     def set_steps_per_launch(self, steps: int) -> None:
         """Time steps per launch (1: one launch per step): in-plane 2D mode, a
         cooperative launch with grid barriers; 2D E_z, temporal blocking on
-        square tiles (16 to 32 nodes a side) with a halo in shared memory (up
-        to 8 steps, 4 in FP64)."""
+        tiles with a halo held in registers (up to 8 steps, 4 in FP64; the
+        default on grids of at most 2^21 nodes, FP64 2^20)."""
         _check(self.lib.fdtd_set_steps_per_launch(self.ctx, int(steps)), "fdtd_set_steps_per_launch")
 
     def set_wavefront(self, steps: int) -> None:

@@ -215,9 +215,9 @@ struct fdtd_ctx {
     // polls a mapped host word the kernel writes and stops enqueuing once it
     // sees this pass's tag (not possible while capturing a graph; the error
     // word still reports the instability).
-    // In-plane 2D contexts: time steps per cooperative launch (1, the
-    // default: two launches per step).
-    int multi_steps = 1;
+    // Time steps per launch as set (fdtd_set_steps_per_launch); 0, the
+    // default: the library's choice for the mode and grid.
+    int multi_steps = 0;
     int guard_every = 256;
     double guard_bound = 0.0;  // 0: automatic, see guard_limit()
     unsigned guard_tag = 0;
@@ -277,6 +277,8 @@ struct fdtd_ctx {
     virtual fdtd_status grayness(double *d_zeta) = 0;
     // L2 residency of the ping-pong state (2D E_z contexts; others ignore it).
     virtual fdtd_status set_l2(double) { return FDTD_OK; }
+    // multi_steps changed.
+    virtual fdtd_status steps_changed() { return FDTD_OK; }
     // New width of the design filter (2D E_z contexts with a filter).
     virtual fdtd_status set_filter_sigma(double) { return FDTD_EINVAL; }
     // Blocks of one step launch and how many take the vector path (2D E_z).
@@ -486,7 +488,15 @@ struct Ctx2D final : fdtd_ctx {
         if (l2) release_l2();
     }
 
+    double l2_req = 0.0;  // the share asked for
     fdtd_status set_l2(double fraction) override
+    {
+        l2_req = fraction;
+        // the blocked launches take no window: nothing is set aside for them
+        return apply_l2(tb_steps() ? 0.0 : fraction);
+    }
+    fdtd_status steps_changed() override { return l2_req > 0 ? apply_l2(tb_steps() ? 0.0 : l2_req) : FDTD_OK; }
+    fdtd_status apply_l2(double fraction)
     {
         for (auto &g : cap)
             if (g.exec) {
@@ -517,11 +527,25 @@ struct Ctx2D final : fdtd_ctx {
     }
     size_t state_bytes = 0;
     long long Mdi = 0;  // pitched design-box elements (dny x dp)
-    // Temporal blocking (kernels_tb2d.cu): with multi_steps > 1 the forward
-    // and the full-history adjoint advance up to min(multi_steps, tb_max)
-    // steps per launch.
-    int tb_max = 0, tb_tile = 32;
-    int tb_steps() const { return (multi_steps > 1 && tb_max > 0) ? std::min(multi_steps, tb_max) : 0; }
+    // Temporal blocking (kernels_rt2d.cu): the forward and the adjoint
+    // advance up to rt_plan().halo steps per launch with multi_steps > 1, or
+    // when it is left automatic (0) and rt_auto says so.
+    bool rt_ok = false, rt_auto = false;
+    int rt_sms = 0;
+    R *rt_coef = nullptr;
+    Rt2DPlan rt_plan() const
+    {
+        Rt2DPlan p = rt2d_plan<R>(geo.nx, geo.ny, rt_sms, multi_steps > 1 ? multi_steps : RT2D_MAX);
+        const long long t32 = (long long)((geo.nx + 31) / 32) * ((geo.ny + 31) / 32);
+        p.form = !(multi_steps > 1 || (sizeof(R) == 4 && t32 <= rt_sms));
+        return p;
+    }
+    int tb_steps() const
+    {
+        if (!rt_ok || (multi_steps == 0 ? !rt_auto : multi_steps == 1)) return 0;
+        const int h = rt_plan().halo;
+        return multi_steps > 1 ? std::min(multi_steps, h) : h;
+    }
     // Steps of the next run from step n (forward): at most T, ending on the
     // guard's multiples while the forward is guarded.
     int tb_run(int n, int end, int T) const
@@ -593,6 +617,7 @@ struct Ctx2D final : fdtd_ctx {
         rho = cv.take<R>(Md);
         rhof = cv.take<R>(Md);
         rho_t = cv.take<R>(Mdi);
+        rt_coef = cv.take<R>(5 * (size_t)Mdi);
         ftmp = cv.take<R>(Md);
         rstage = cv.take<R>(Md);
         G = cv.take<double>(Mdi);
@@ -640,19 +665,19 @@ struct Ctx2D final : fdtd_ctx {
         FDTD_TRY(upload_filter(c.filter_sigma));
         launch_zero_bytes(err, 4 * sizeof(unsigned), st);
         ++launches;
-        tb_max = tb2d_max_steps<R>();
-        // Default: temporal blocking on FP32 grids of at most one 32 x 32 tile
-        // per SM, where the launch-per-step kernels are single partial waves
-        // (measured: 316^2, 7.1 -> 3.4 us per forward step with 32 x 32
-        // tiles); larger or FP64 grids run faster one launch per step.  The
-        // tile side is the smallest whose tiles still fit one wave.
+        rt_ok = rt2d_ready<R>();
         {
-            int dev = 0, sms = 0;
+            int dev = 0;
             cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            tb_tile = tb2d_tile(c.nx, c.ny, sms);
-            const long long tiles = (long long)((c.nx + tb_tile - 1) / tb_tile) * ((c.ny + tb_tile - 1) / tb_tile);
-            if (sizeof(R) == 4 && tb_max > 0 && tiles <= sms) multi_steps = TB_MAX;
+            cudaDeviceGetAttribute(&rt_sms, cudaDevAttrMultiProcessorCount, dev);
+            // Measured, launch per step against blocked (us per forward /
+            // full-history adjoint step): FP32 316^2 6.9 / 7.5 against 1.02 /
+            // 1.28, 500^2 7.5 / 7.6 against 2.1 / 2.3, 1000^2 10.6 / 10.4
+            // against 5.7 / 6.5, 1400^2 13.1 / 15.3 against 10.1 / 11.6, 2048^2
+            // 23.8 / 27.7 against 21.7 / 24.7 (but 21.2 with the L2 window,
+            // which the blocked launches do not take); FP64 160^2 12.1 / 15.1
+            // against 3.3 / 3.3, 1000^2 52 / 72 against 49 / 53.
+            rt_auto = ncells <= (sizeof(R) == 4 ? 1LL << 21 : 1LL << 20);
         }
         return cuda_ok(cudaStreamSynchronize(st));
     }
@@ -702,7 +727,7 @@ struct Ctx2D final : fdtd_ctx {
     fdtd_status forward(double *d_W) override
     {
         FDTD_TRY(cuda_ok(upload_coef_2d<R>(coef_slot, coef(), stream)));
-        if (tb_steps()) FDTD_TRY(cuda_ok(upload_coef_tb2d<R>(coef_slot, coef(), stream)));
+        if (tb_steps()) FDTD_TRY(cuda_ok(upload_coef_rt2d<R>(coef_slot, coef(), stream)));
         int keepA = curA;
         FDTD_TRY(run_pass(this, 0, curF, keepA, [&] { return enqueue_forward(); }));
         if (d_W && d_W != misc)
@@ -713,7 +738,7 @@ struct Ctx2D final : fdtd_ctx {
     fdtd_status adjoint() override
     {
         FDTD_TRY(cuda_ok(upload_coef_2d<R>(coef_slot, coef(), stream)));
-        if (tb_steps()) FDTD_TRY(cuda_ok(upload_coef_tb2d<R>(coef_slot, coef(), stream)));
+        if (tb_steps()) FDTD_TRY(cuda_ok(upload_coef_rt2d<R>(coef_slot, coef(), stream)));
         return run_pass(this, 1, curF, curA, [&] { return enqueue_adjoint(); });
     }
 
@@ -746,6 +771,18 @@ struct Ctx2D final : fdtd_ctx {
         return FDTD_OK;
     }
 
+    Rt2D<R> rt_args(const Rt2DPlan &pl) const
+    {
+        Rt2D<R> w{};
+        w.halo = pl.halo;
+        w.tw = pl.tw;
+        w.th = pl.th;
+        w.Mdi = Mdi;
+        w.coef = rt_coef;
+        w.kappa1 = cfg.pml_kappa_max == 1.0;
+        return w;
+    }
+
     // Advance the forward state from step n0 by count steps.  gap: record
     // E^{n+1} of the gap; rec_base: record design-box E^{n+1} in slot
     // (n - n0) of rec_base (null: no record).
@@ -754,18 +791,17 @@ struct Ctx2D final : fdtd_ctx {
         Step2D<R> a{};
         a.rho_t = rho_t;
         if (const int T = tb_steps()) {
+            const Rt2DPlan pl = rt_plan();
             for (int n = n0; n < n0 + count;) {
-                Tb2D<R> w{};
+                Rt2D<R> w = rt_args(pl);
                 w.count = tb_run(n, n0 + count, T);
-                w.tile = tb_tile;
                 w.n0 = n;
+                w.first = n == n0;
                 w.rec0 = n0;
-                w.Mdi = Mdi;
                 w.src = src_tab;
                 w.gap = (gap && Mg) ? gap_hist : nullptr;
                 w.rec = rec_base;
-                w.rho_t = rho_t;
-                launches += launch_tb2d<R>(0, geo, F[curF], F[curF ^ 1], coef_slot, px, py, w, stream);
+                launches += launch_rt2d<R>(0, geo, F[curF], F[curF ^ 1], coef_slot, px, py, w, pl, stream);
                 curF ^= 1;
                 cell_updates += (long long)w.count * ncells;
                 n += w.count;
@@ -792,18 +828,17 @@ struct Ctx2D final : fdtd_ctx {
         a.rho_t = rho_t;
         a.G = G;
         if (const int T = tb_steps()) {
+            const Rt2DPlan pl = rt_plan();
             for (int m = m_hi; m > m_lo;) {
-                Tb2D<R> w{};
+                Rt2D<R> w = rt_args(pl);
                 w.count = std::min(T, m - m_lo);
-                w.tile = tb_tile;
                 w.n0 = m;
+                w.first = m == m_hi;
                 w.rec0 = slot0;
-                w.Mdi = Mdi;
                 w.gap = Mg ? gap_hist : nullptr;
                 w.rec = base;
-                w.rho_t = rho_t;
                 w.G = G;
-                launches += launch_tb2d<R>(1, geo, A[curA], A[curA ^ 1], coef_slot, px, py, w, stream);
+                launches += launch_rt2d<R>(1, geo, A[curA], A[curA ^ 1], coef_slot, px, py, w, pl, stream);
                 curA ^= 1;
                 m -= w.count;
             }
@@ -834,6 +869,7 @@ struct Ctx2D final : fdtd_ctx {
         launch_zero_bytes(F_base[1], state_bytes, st);
         if (Mg) launch_zero_bytes(gap_hist, Mg * sizeof(R), st);
         launches += 3;
+        if (tb_steps()) launches += launch_rt2d_coef<R>(geo, coef_slot, rho_t, rt_coef, Mdi, st);
         guarding = true;
         if (K <= 0) {
             advance_forward(0, N, true, rec);
@@ -863,6 +899,7 @@ struct Ctx2D final : fdtd_ctx {
         launch_zero_bytes(A_base[1], state_bytes, st);
         launch_zero_bytes(G, Mdi * sizeof(double), st);
         launches += 3;
+        if (tb_steps()) launches += launch_rt2d_coef<R>(geo, coef_slot, rho_t, rt_coef, Mdi, st);
         if (K <= 0) {
             advance_adjoint(N, 0, 0);
             return check_launch();
@@ -1969,7 +2006,7 @@ fdtd_status fdtd_set_steps_per_launch(fdtd_ctx *ctx, int steps)
     if (!ctx || steps < 1 || steps > 4096) return FDTD_EINVAL;
     ctx->multi_steps = steps;
     ctx->drop_graphs();  // captured passes hold the old launches
-    return FDTD_OK;
+    return ctx->steps_changed();
 }
 
 fdtd_status fdtd_set_wavefront(fdtd_ctx *ctx, int steps)

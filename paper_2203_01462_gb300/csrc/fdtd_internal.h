@@ -92,6 +92,20 @@ template <typename R>
 int launch_step2d(int mode, const Geo2D &g, const State2D<R> &in, const State2D<R> &out, int coef_slot,
                   const Pml1D<R> &px, const Pml1D<R> &py, const Step2D<R> &a, cudaStream_t st, const cudaAccessPolicyWindow *win);
 
+// Tile of the 2D step kernel's blocks (nodes), its vector path's predicate
+// for the tile at (x0, y0) (none of the nodes it reads is a wall or CPML
+// node), and whether such a tile has design, gap or (forward) source nodes.
+constexpr int STEP2D_TX = 128, STEP2D_TY = 4;
+__host__ __device__ __forceinline__ bool step2d_vector_tile(int nx, int ny, int np, int x0, int y0)
+{
+    return x0 - 1 >= np + 1 && x0 + STEP2D_TX <= nx - np - 2 && y0 - 1 >= np + 1 && y0 + STEP2D_TY <= ny - np - 2;
+}
+__host__ __device__ __forceinline__ bool step2d_touches(const Geo2D &g, int mode, int x0, int y0)
+{
+    return (x0 < g.dx0 + g.dnx && x0 + STEP2D_TX > g.dx0 && y0 < g.dy0 + g.dny && y0 + STEP2D_TY > g.dy0) ||
+           (mode == 0 && x0 < g.sx1 && x0 + STEP2D_TX > g.sx0 && y0 < g.sy1 && y0 + STEP2D_TY > g.sy0);
+}
+
 // Blocks of one 2D step launch, and how many of them take the vector path.
 void step2d_block_counts(const Geo2D &g, long long *total, long long *vector);
 
@@ -251,36 +265,46 @@ template <typename R>
 int launch_step3d(int mode, const Geo3D &g, const State3D<R> &s, int coef_slot, const Pml3D<R> &pm,
                   const Step3D<R> &a, cudaStream_t st);
 
-// Temporally blocked 2D E_z steps (kernels_tb2d.cu): a block owns a square
-// tile (`tile` nodes a side, tb2d_tile) and advances count <= TB_MAX steps
-// on it and a halo of count nodes in shared memory, reading state `in` and
-// writing its tile into `out`.
+// Temporally blocked 2D E_z steps with the tile in registers
+// (kernels_rt2d.cu): a block owns tw x th nodes with a halo and advances
+// count <= halo <= RT2D_MAX steps, reading state `in` and writing its tile
+// into `out`.
 // Forward: steps n0 .. n0+count-1 (source row n, gap row n+1, design record
 // slot n - rec0); adjoint: m = n0 down to n0-count+1 (gap row m, record slot
-// m-1-rec0), G the accumulator.
-constexpr int TB_MAX = 8;
+// m-1-rec0), G the accumulator.  coef: five arrays of Mdi words, the Drude
+// coefficients of rho~ (launch_rt2d_coef, once per pass).
+constexpr int RT2D_MAX = 8;
 template <typename R>
-struct Tb2D {
-    int count, n0, rec0, tile;
+struct Rt2D {
+    int count, n0, rec0;
+    int halo, tw, th;
+    int first;      // first launch of a run: everything waits for the kernel before it
+    int kappa1;     // every CPML kappa is 1
     long long Mdi;
     const R *src;
     R *gap;
     R *rec;
-    const R *rho_t;
+    const R *coef;
     double *G;
 };
-size_t tb2d_smem_bytes(int esz, int T);
-// Tile side of the blocked kernel for an nx x ny grid on `sms` SMs.
-int tb2d_tile(int nx, int ny, int sms);
-// The most steps per launch whose region fits a block's shared memory (and
-// the kernels' shared-memory limit raised to it), or 0.
+// Halo, tile sides, warps per block, blocks along x and y, and the rounding
+// form of the Drude update (kernels_rt2d.cu, FORM).
+struct Rt2DPlan {
+    int halo, tw, th, nw, bx, by, form;
+};
 template <typename R>
-int tb2d_max_steps();
+Rt2DPlan rt2d_plan(int nx, int ny, int sms, int steps);
+// Raises the kernels' shared-memory limit on the current device; false if
+// they cannot run there.
 template <typename R>
-int launch_tb2d(int mode, const Geo2D &g, const State2D<R> &in, const State2D<R> &out, int coef_slot,
-                const Pml1D<R> &px, const Pml1D<R> &py, const Tb2D<R> &w, cudaStream_t st);
+bool rt2d_ready();
 template <typename R>
-cudaError_t upload_coef_tb2d(int slot, const Coef<R> &c, cudaStream_t st);
+int launch_rt2d(int mode, const Geo2D &g, const State2D<R> &in, const State2D<R> &out, int coef_slot,
+                const Pml1D<R> &px, const Pml1D<R> &py, const Rt2D<R> &w, const Rt2DPlan &p, cudaStream_t st);
+template <typename R>
+int launch_rt2d_coef(const Geo2D &g, int coef_slot, const R *rho_t, R *coef, long long Mdi, cudaStream_t st);
+template <typename R>
+cudaError_t upload_coef_rt2d(int slot, const Coef<R> &c, cudaStream_t st);
 
 // Several 3D steps in one persistent launch (kernels_3d.cu, k_wave3d).
 // The grid is cut into z slabs of two planes; an item is up to `tpi`

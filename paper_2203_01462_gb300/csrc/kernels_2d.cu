@@ -32,16 +32,9 @@ namespace {
 
 constexpr int BX = 32, BY = 4, VX = 4;
 constexpr int TILE_X = BX * VX;
+static_assert(TILE_X == STEP2D_TX && BY == STEP2D_TY, "the shared tile predicates are this kernel's");
 
 __device__ __forceinline__ bool in_range(int v, int lo, int n) { return (unsigned)(v - lo) < (unsigned)n; }
-
-// Vector path for blocks none of whose read nodes (x0-1 .. x0+TILE_X,
-// y0-1 .. y0+BY) is a wall or CPML node (uniform across the block).  The
-// host counts blocks with the same predicate (step2d_block_counts).
-__host__ __device__ __forceinline__ bool vector_tile(int nx, int ny, int np, int x0, int y0)
-{
-    return x0 - 1 >= np + 1 && x0 + TILE_X <= nx - np - 2 && y0 - 1 >= np + 1 && y0 + BY <= ny - np - 2;
-}
 
 // Programmatic dependent launch: the step kernels are launched with
 // programmatic stream serialisation, so a step's blocks may be scheduled
@@ -207,7 +200,7 @@ __device__ __forceinline__ void step2d_body(const Geo2D &g, const State2D<R> &in
     const int nx = g.nx, ny = g.ny, np = g.npml, P = g.px;
     const R S = c.S;
 
-    if (vector_tile(nx, ny, np, x0, y0)) {
+    if (step2d_vector_tile(nx, ny, np, x0, y0)) {
         const int q = j * P + i0;
         R e[4], eN[4], eS[4], hx[4], hxS[4], hy[4];
         ld4(in.Ez + q, e);
@@ -230,8 +223,7 @@ __device__ __forceinline__ void step2d_body(const Geo2D &g, const State2D<R> &in
 #pragma unroll
         for (int k = 0; k < 4; ++k) curlS[k] += yn[k + 1] - yn[k];
 
-        const bool touches = (x0 < g.dx0 + g.dnx && x0 + TILE_X > g.dx0 && y0 < g.dy0 + g.dny && y0 + BY > g.dy0) ||
-                             (MODE == 0 && x0 < g.sx1 && x0 + TILE_X > g.sx0 && y0 < g.sy1 && y0 + BY > g.sy0);
+        const bool touches = step2d_touches(g, MODE, x0, y0);
         if (!touches) {
             const R Se = S * c.inv_eps_s;
 #pragma unroll
@@ -332,7 +324,7 @@ void step2d_block_counts(const Geo2D &g, long long *total, long long *vector)
     const int gx = (g.nx + TILE_X - 1) / TILE_X, gy = (g.ny + BY - 1) / BY;
     long long v = 0;
     for (int by = 0; by < gy; ++by)
-        for (int bx = 0; bx < gx; ++bx) v += vector_tile(g.nx, g.ny, g.npml, bx * TILE_X, by * BY) ? 1 : 0;
+        for (int bx = 0; bx < gx; ++bx) v += step2d_vector_tile(g.nx, g.ny, g.npml, bx * TILE_X, by * BY) ? 1 : 0;
     *total = (long long)gx * gy;
     *vector = v;
 }
