@@ -251,13 +251,17 @@ fdtd_status fdtd_set_stability_guard(fdtd_ctx *ctx, int every, double max_abs);
 fdtd_status fdtd_set_filter_width(fdtd_ctx *ctx, double sigma);
 
 /* Time steps per launch.  In-plane 2D contexts (pol = FDTD_POL_INPLANE):
- * default 1 (one launch per half step).  With more than one, a run of
- * steps is one cooperative launch, one block per SM, whose half steps are
+ * left unset, up to 8 steps per launch (4 in FP64) by temporal blocking, as
+ * for E_z below (the paper's 291^2 and 491^2 geometries: 4.9 and 5.9 us per
+ * forward step with one launch per half step, 1.4 and 2.3 blocked; the
+ * adjoint's sensitivities are summed by a second kernel from the records of
+ * up to 32 steps).  1: one launch per half step.  With more than one, a run
+ * of steps is one cooperative launch, one block per SM, whose half steps are
  * separated by grid-wide barriers with bounded waits (FDTD_ETIMEOUT from
- * fdtd_sync if one gives up).  Results are bit-identical either way.  On a
- * GB300 the barrier costs more than the launch boundary it replaces (about
- * 12 against 6 us per step on the paper's 491^2 geometry), hence the
- * default.  Such passes are not replayed as CUDA graphs.
+ * fdtd_sync if one gives up), about 12 us per 491^2 step; such passes are not
+ * replayed as CUDA graphs.  W~ and the gap history are bit-identical in all
+ * three (up to rounding with pml_kappa_max other than 1, or a Courant number
+ * that is not a power of two); the gradient agrees to 1e-12.
  *
  * 2D E_z contexts: with steps > 1 the forward (and recompute) and the
  * adjoint advance up to min(steps, 8) steps per launch (4 in FP64, and 4 to 8

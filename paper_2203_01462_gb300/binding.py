@@ -297,10 +297,11 @@ class Solver:
         self.w["filter_sigma"] = float(sigma)
 
     def set_steps_per_launch(self, steps: int) -> None:
-        """Time steps per launch (1: one launch per step): in-plane 2D mode, a
-        cooperative launch with grid barriers; 2D E_z, temporal blocking on
-        tiles with a halo held in registers (up to 8 steps, 4 in FP64; the
-        default on grids of at most 2^21 nodes, FP64 2^20)."""
+        """Time steps per launch.  Left unset: temporal blocking on tiles with a
+        halo held in registers (up to 8 steps, 4 in FP64; E_z grids of at most
+        2^21 nodes, FP64 2^20, and all in-plane grids).  1: one launch per step
+        (in-plane: per half step).  More: E_z, blocked with at most that many
+        steps; in-plane, a cooperative launch with grid barriers."""
         _check(self.lib.fdtd_set_steps_per_launch(self.ctx, int(steps)), "fdtd_set_steps_per_launch")
 
     def set_wavefront(self, steps: int) -> None:

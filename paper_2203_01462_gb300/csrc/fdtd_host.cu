@@ -1052,8 +1052,32 @@ long long edge_total(const int *lo, const int *hi)
 template <typename R>
 struct CtxP final : fdtd_ctx {
     GeoP geo{};
-    StateP<R> F{}, A{};  // updated in place (split H and E launches)
-    char *F_base = nullptr, *A_base = nullptr;
+    // Ping-pong pairs for the blocked launches; the split H and E launches and
+    // the multi-step launch update buffer curF / curA in place.
+    StateP<R> F[2]{}, A[2]{};
+    char *F_base[2] = {nullptr, nullptr}, *A_base[2] = {nullptr, nullptr};
+    int curF = 0, curA = 0;
+    // Temporal blocking (kernels_rt2dp.cu), the default (steps per launch not
+    // set) where it was measured faster.
+    bool rt_ok = false;
+    int rt_sms = 0;
+    R *rt_coef[2] = {nullptr, nullptr};
+    bool rt() const { return rt_ok && multi_steps == 0; }
+    Rt2DPlan rt_plan() const { return rt2dp_plan<R>(geo.nx, geo.ny, rt_sms); }
+    // Adjoint records of a chunk of steps, and the adjoint J and E before it.
+    R *arec = nullptr, *jsens[2] = {nullptr, nullptr}, *eprev[2] = {nullptr, nullptr};
+    RtP<R> rt_args(const Rt2DPlan &pl) const
+    {
+        RtP<R> w{};
+        w.halo = pl.halo;
+        w.tw = pl.tw;
+        w.th = pl.th;
+        w.kappa1 = cfg.pml_kappa_max == 1.0;
+        w.rec_step = Mdi_all();
+        w.coef[0] = rt_coef[0];
+        w.coef[1] = rt_coef[1];
+        return w;
+    }
     size_t state_bytes = 0;
     long long Mdx = 0;  // design entries of the E_x edges (first part of rho)
     R *rho = nullptr, *rho_t[2] = {nullptr, nullptr}, *rstage = nullptr;
@@ -1159,11 +1183,17 @@ struct CtxP final : fdtd_ctx {
             geo.s1[a] = c.src_hi[a];
         }
         const long long N = c.nsteps;
-        carve_state(cv, F, F_base);
-        carve_state(cv, A, A_base);
+        for (int b = 0; b < 2; ++b) carve_state(cv, F[b], F_base[b]);
+        for (int b = 0; b < 2; ++b) carve_state(cv, A[b], A_base[b]);
         rho = cv.take<R>(Md);
         rho_t[0] = cv.take<R>((size_t)geo.Mdi[0]);
         rho_t[1] = cv.take<R>((size_t)geo.Mdi[1]);
+        for (int cc = 0; cc < 2; ++cc) rt_coef[cc] = cv.take<R>(5 * (size_t)geo.Mdi[cc]);
+        arec = cv.take<R>((size_t)RT2DP_CHUNK * Mdi_all());
+        for (int cc = 0; cc < 2; ++cc) {
+            jsens[cc] = cv.take<R>((size_t)geo.Mdi[cc]);
+            eprev[cc] = cv.take<R>((size_t)geo.Mdi[cc]);
+        }
         rstage = cv.take<R>(Md);
         G[0] = cv.take<double>((size_t)geo.Mdi[0]);
         G[1] = cv.take<double>((size_t)geo.Mdi[1]);
@@ -1206,6 +1236,12 @@ struct CtxP final : fdtd_ctx {
         launch_zero_bytes(err, 4 * sizeof(unsigned), st);
         ++launches;
         multi_fits = stepp_multi_fits<R>(geo);
+        rt_ok = rt2dp_ready<R>();
+        {
+            int dev = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&rt_sms, cudaDevAttrMultiProcessorCount, dev);
+        }
         return cuda_ok(cudaStreamSynchronize(st));
     }
 
@@ -1214,8 +1250,9 @@ struct CtxP final : fdtd_ctx {
     fdtd_status forward(double *d_W) override
     {
         FDTD_TRY(cuda_ok(upload_coef_p<R>(coef_slot, coef(), stream)));
-        int f = 0, a = 0;
-        FDTD_TRY(run_pass(this, 0, f, a, [&] { return enqueue_forward(); }));
+        if (rt()) FDTD_TRY(cuda_ok(upload_coef_rt2dp<R>(coef_slot, coef(), stream)));
+        int keepA = curA;
+        FDTD_TRY(run_pass(this, 0, curF, keepA, [&] { return enqueue_forward(); }));
         if (d_W && d_W != misc)
             FDTD_TRY(cuda_ok(cudaMemcpyAsync(d_W, misc, sizeof(double), cudaMemcpyDeviceToDevice, stream)));
         return check_launch();
@@ -1224,8 +1261,8 @@ struct CtxP final : fdtd_ctx {
     fdtd_status adjoint() override
     {
         FDTD_TRY(cuda_ok(upload_coef_p<R>(coef_slot, coef(), stream)));
-        int f = 0, a = 0;
-        return run_pass(this, 1, f, a, [&] { return enqueue_adjoint(); });
+        if (rt()) FDTD_TRY(cuda_ok(upload_coef_rt2dp<R>(coef_slot, coef(), stream)));
+        return run_pass(this, 1, curF, curA, [&] { return enqueue_adjoint(); });
     }
     fdtd_status check_launch() { return cuda_ok(cudaGetLastError()); }
 
@@ -1258,6 +1295,26 @@ struct CtxP final : fdtd_ctx {
 
     void advance_forward(int n0, int count, bool gap, R *rec_base)
     {
+        if (rt()) {
+            const Rt2DPlan pl = rt_plan();
+            for (int n = n0; n < n0 + count;) {
+                int end = n0 + count;
+                if (guarding && guard_every > 0) end = std::min(end, (n / guard_every + 1) * guard_every);
+                RtP<R> w = rt_args(pl);
+                w.count = std::min(pl.halo, end - n);
+                w.n0 = n;
+                w.first = n == n0;
+                w.src = src_tab;
+                w.gap = (gap && Mg) ? gap_hist : nullptr;
+                w.rec = rec_base ? rec_base + (size_t)(n - n0) * Mdi_all() : nullptr;
+                launches += launch_rt2dp<R>(0, geo, F[curF], F[curF ^ 1], coef_slot, pm, w, pl, stream);
+                curF ^= 1;
+                cell_updates += (long long)w.count * ncells;
+                n += w.count;
+                if (guard_after<R>(n, F_base[curF], state_bytes)) break;
+            }
+            return;
+        }
         if (multi()) {
             // runs of steps that end on multiples of chunk(), which divides
             // the guard interval, so the guard sees every step it checks
@@ -1274,9 +1331,9 @@ struct CtxP final : fdtd_ctx {
                 pl.rec0 = n0;
                 pl.n0 = n;
                 pl.count = n1 - n;
-                launch_multi(0, F, pl);
+                launch_multi(0, F[curF], pl);
                 n = n1;
-                if (guard_after<R>(n, F_base, state_bytes)) break;
+                if (guard_after<R>(n, F_base[curF], state_bytes)) break;
             }
             return;
         }
@@ -1287,14 +1344,37 @@ struct CtxP final : fdtd_ctx {
             R *slot = rec_base ? rec_base + (size_t)(n - n0) * Mdi_all() : nullptr;
             a.rec[0] = slot;
             a.rec[1] = slot ? slot + geo.Mdi[0] : nullptr;
-            launches += launch_stepp<R>(0, geo, F, coef_slot, pm, a, stream);
+            launches += launch_stepp<R>(0, geo, F[curF], coef_slot, pm, a, stream);
             cell_updates += ncells;
-            if (guard_after<R>(n + 1, F_base, state_bytes)) break;
+            if (guard_after<R>(n + 1, F_base[curF], state_bytes)) break;
         }
     }
 
     void advance_adjoint(int m_hi, int m_lo, int slot0)
     {
+        if (rt()) {
+            const Rt2DPlan pl = rt_plan();
+            for (int c_hi = m_hi; c_hi > m_lo;) {  // chunks of adjoint steps, then their sensitivities
+                const int c_lo = std::max(m_lo, c_hi - RT2DP_CHUNK);
+                for (int m = c_hi; m > c_lo;) {
+                    RtP<R> w = rt_args(pl);
+                    w.count = std::min(pl.halo, m - c_lo);
+                    w.n0 = m;
+                    w.first = m == c_hi;
+                    w.gap = Mg ? gap_hist : nullptr;
+                    w.rec = arec + (size_t)(c_hi - m) * Mdi_all();
+                    launches += launch_rt2dp<R>(1, geo, A[curA], A[curA ^ 1], coef_slot, pm, w, pl, stream);
+                    curA ^= 1;
+                    m -= w.count;
+                }
+                launches += launch_rt2dp_sens<R>(geo, coef_slot, rt_coef, Mdi_all(), arec,
+                                                 rec + (size_t)(c_hi - 1 - slot0) * Mdi_all(), c_hi - c_lo, jsens, eprev, G,
+                                                 stream);
+                c_hi = c_lo;
+            }
+            cell_updates += (long long)(m_hi - m_lo) * ncells;
+            return;
+        }
         if (multi()) {
             for (int m = m_hi; m > m_lo;) {
                 const int cnt = std::min(multi_steps, m - m_lo);
@@ -1307,7 +1387,7 @@ struct CtxP final : fdtd_ctx {
                 pl.rec0 = slot0;
                 pl.n0 = m;
                 pl.count = cnt;
-                launch_multi(1, A, pl);
+                launch_multi(1, A[curA], pl);
                 m -= cnt;
             }
             return;
@@ -1320,7 +1400,7 @@ struct CtxP final : fdtd_ctx {
             R *slot = rec + (size_t)(m - 1 - slot0) * Mdi_all();
             a.rec[0] = slot;
             a.rec[1] = slot + geo.Mdi[0];
-            launches += launch_stepp<R>(1, geo, A, coef_slot, pm, a, stream);
+            launches += launch_stepp<R>(1, geo, A[curA], coef_slot, pm, a, stream);
         }
         cell_updates += (long long)(m_hi - m_lo) * ncells;
     }
@@ -1329,9 +1409,15 @@ struct CtxP final : fdtd_ctx {
     {
         cudaStream_t st = stream;
         const int N = cfg.nsteps, K = cfg.snapshot_every;
-        launch_zero_bytes(F_base, state_bytes, st);
+        curF = 0;
+        launch_zero_bytes(F_base[0], state_bytes, st);
         if (Mg) launch_zero_bytes(gap_hist, Mg * sizeof(R), st);
         launches += 2;
+        if (rt()) {
+            // words the blocked launches never write (padding, walls' psi) are zero in both buffers
+            launch_zero_bytes(F_base[1], state_bytes, st);
+            launches += 1 + launch_rt2dp_coef<R>(geo, coef_slot, rho_t, rt_coef, st);
+        }
         if (multi()) reset_coop();
         guarding = true;
         if (K <= 0) {
@@ -1340,7 +1426,7 @@ struct CtxP final : fdtd_ctx {
             for (int s = 0; s < nsnap; ++s) {
                 if (guard_stop) break;
                 const int n0 = s * K, cnt = std::min(K, N - n0);
-                snapshot_save<R>(cfg.snapshot_dtype, F_base, state_bytes, snaps + (size_t)s * snap_stride, st);
+                snapshot_save<R>(cfg.snapshot_dtype, F_base[curF], state_bytes, snaps + (size_t)s * snap_stride, st);
                 ++launches;
                 advance_forward(n0, cnt, true, nullptr);
             }
@@ -1357,17 +1443,26 @@ struct CtxP final : fdtd_ctx {
     {
         cudaStream_t st = stream;
         const int N = cfg.nsteps, K = cfg.snapshot_every;
-        launch_zero_bytes(A_base, state_bytes, st);
+        curA = 0;
+        launch_zero_bytes(A_base[0], state_bytes, st);
         launch_zero_bytes(G[0], geo.Mdi[0] * sizeof(double), st);
         launch_zero_bytes(G[1], geo.Mdi[1] * sizeof(double), st);
         launches += 3;
+        if (rt()) {
+            launch_zero_bytes(A_base[1], state_bytes, st);
+            for (int cc = 0; cc < 2; ++cc) {
+                launch_zero_bytes(jsens[cc], geo.Mdi[cc] * sizeof(R), st);
+                launch_zero_bytes(eprev[cc], geo.Mdi[cc] * sizeof(R), st);
+            }
+            launches += 5 + launch_rt2dp_coef<R>(geo, coef_slot, rho_t, rt_coef, st);
+        }
         if (multi()) reset_coop();
         if (K <= 0) {
             advance_adjoint(N, 0, 0);
         } else {
             for (int s = nsnap - 1; s >= 0; --s) {
                 const int n0 = s * K, n1 = std::min(n0 + K, N);
-                snapshot_load<R>(cfg.snapshot_dtype, snaps + (size_t)s * snap_stride, F_base, state_bytes, st);
+                snapshot_load<R>(cfg.snapshot_dtype, snaps + (size_t)s * snap_stride, F_base[curF], state_bytes, st);
                 ++launches;
                 advance_forward(n0, n1 - n0, false, rec);
                 advance_adjoint(n1, n0, n0);

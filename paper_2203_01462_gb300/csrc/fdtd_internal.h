@@ -306,6 +306,40 @@ int launch_rt2d_coef(const Geo2D &g, int coef_slot, const R *rho_t, R *coef, lon
 template <typename R>
 cudaError_t upload_coef_rt2d(int slot, const Coef<R> &c, cudaStream_t st);
 
+// Temporally blocked in-plane steps (kernels_rt2dp.cu); as Rt2D.  Both runs
+// record the design edges' E of their steps in consecutive slots from rec on
+// (or not: null), rec_step words each, Ex part first.
+template <typename R>
+struct RtP {
+    int count, n0;
+    int halo, tw, th;
+    int first, kappa1;
+    long long rec_step;
+    const R *src;
+    R *gap;
+    R *rec;
+    const R *coef[2];
+};
+// Adjoint steps whose records are kept before their sensitivities are summed.
+constexpr int RT2DP_CHUNK = 32;
+// The sums of `count` steps: adjoint records ae (ascending slots), forward
+// records fe (descending), step words apart; jsens and eprev carry the
+// adjoint J and E from one call to the next.
+template <typename R>
+int launch_rt2dp_sens(const GeoP &g, int coef_slot, const R *const coef[2], long long step, const R *ae, const R *fe,
+                      int count, R *const jsens[2], R *const eprev[2], double *const G[2], cudaStream_t st);
+template <typename R>
+Rt2DPlan rt2dp_plan(int nx, int ny, int sms);
+template <typename R>
+bool rt2dp_ready();
+template <typename R>
+int launch_rt2dp(int mode, const GeoP &g, const StateP<R> &in, const StateP<R> &out, int coef_slot,
+                 const PmlP<R> &pm, const RtP<R> &w, const Rt2DPlan &p, cudaStream_t st);
+template <typename R>
+int launch_rt2dp_coef(const GeoP &g, int coef_slot, const R *const rho_t[2], R *const coef[2], cudaStream_t st);
+template <typename R>
+cudaError_t upload_coef_rt2dp(int slot, const Coef<R> &c, cudaStream_t st);
+
 // Several 3D steps in one persistent launch (kernels_3d.cu, k_wave3d).
 // The grid is cut into z slabs of two planes; an item is up to `tpi`
 // x-adjacent node tiles of one row of one slab, and a job is every item of

@@ -41,46 +41,11 @@
 #include <type_traits>
 
 #include "coef_slots.cuh"
-#include "fdtd_internal.h"
-#include "launch.cuh"
+#include "rt_common.cuh"
 
 namespace fdtd {
 
 namespace {
-
-__device__ __forceinline__ bool in_range(int v, int lo, int n) { return (unsigned)(v - lo) < (unsigned)n; }
-__device__ __forceinline__ float rcp(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double rcp(double x) { return __drcp_rn(x); }
-
-// Slab indices of the CPML arrays (E: node positions, H: half positions); -1 outside.
-__device__ __forceinline__ int slab_e(int p, int n, int np) { return p < np ? p : (p >= n - np ? p - (n - 2 * np) : -1); }
-__device__ __forceinline__ int slab_h(int p, int n, int np)
-{
-    return p < np ? p : ((p >= n - 1 - np && p < n - 1) ? np + p - (n - 1 - np) : -1);
-}
-
-// VX adjacent words as one access (VX sizeof(R) = 8 bytes).
-__device__ __forceinline__ void ldv(const float *p, float (&o)[2])
-{
-    const float2 t = *reinterpret_cast<const float2 *>(p);
-    o[0] = t.x; o[1] = t.y;
-}
-__device__ __forceinline__ void stv(float *p, const float (&o)[2]) { *reinterpret_cast<float2 *>(p) = make_float2(o[0], o[1]); }
-__device__ __forceinline__ void ldv(const double *p, double (&o)[1]) { o[0] = *p; }
-__device__ __forceinline__ void stv(double *p, const double (&o)[1]) { *p = o[0]; }
-template <typename R, int VX>
-__device__ __forceinline__ void zero(R (&o)[VX])
-{
-#pragma unroll
-    for (int v = 0; v < VX; ++v) o[v] = R(0);
-}
-
-// 8-byte asynchronous copy to shared memory.
-__device__ __forceinline__ void cp8(void *s, const void *g)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(s)), "l"(g)
-                 : "memory");
-}
 
 // Shape per precision: VX columns per lane, RPW rows per warp.
 template <typename R>
@@ -106,33 +71,6 @@ __host__ __device__ size_t smem_words(int nw, int count, int gapw, int mode)
 
 // Largest gap whose adjoint source is staged in shared memory (nodes).
 constexpr int GAP_STAGED = 256;
-
-// Exact sum of a few FP32 products as an unevaluated FP32 pair (hi + lo):
-// the adjoint's sensitivity sum of one launch.  A GB300 runs FP64 (and
-// conversions to it) at 1/64 of the FP32 rate, so one FP64 product and sum
-// per node and step (0.7 of 2.3 us per 316^2 adjoint step) becomes twelve
-// FP32 operations, and one FP64 addition per node and launch.  The product's
-// rounding error is recovered by an FMA and the sum's by Knuth's two-sum.
-struct Pair {
-    float hi, lo;
-    // The product's error would be lost: it is not zero and below 2^-100, or
-    // it is beyond 2^126 (or not a number).
-    static __device__ __forceinline__ bool far(float a, float b)
-    {
-        const float p = fabsf(__fmul_rn(a, b));
-        return (p < 0x1p-100f && a != 0.0f && b != 0.0f) || !(p <= 0x1p126f);
-    }
-    static __device__ __forceinline__ bool far(double, double) { return false; }
-    __device__ __forceinline__ void add(double, double) {}
-    __device__ __forceinline__ void add(float a, float b)
-    {
-        const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
-        const float s = __fadd_rn(hi, p), t = __fsub_rn(s, hi);
-        const float r = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(p, t));
-        hi = s;
-        lo = __fadd_rn(lo, __fadd_rn(r, e));
-    }
-};
 
 // FORM: which product of a Drude node's E update is rounded before the sum,
 // ca E (1) or cb (curl - ...) (0).  Grids small enough for one 32 x 32 tile
@@ -164,7 +102,9 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
     R *yt = xt + 6 * W;                    // [6][YT]: the same of the rows, entry 0 = the row below the region
     R *ssrc = yt + 6 * YT;
     R *sgap = ssrc + RT2D_MAX;
-    const bool gstage = MODE == 1 && Mg <= GAP_STAGED;
+    // the gap's adjoint source is staged by the blocks whose region holds gap nodes
+    const bool gstage = MODE == 1 && Mg <= GAP_STAGED && w.gap && xr < g.gx0 + g.gnx && xr + W > g.gx0 &&
+                        yr < g.gy0 + g.gny && yr + nw * RPW > g.gy0;
     R *srec = sgap + (gstage ? ((T * Mg + 1) & ~1) : 0);  // [T][RPW][threads][VX], 8-byte aligned
 
     // The region meets the absorbing layer of the columns / rows.
@@ -202,8 +142,8 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
             yt[5 * YT + q] = hs ? py.kiH[p] : R(1);
         }
     if (MODE == 0 && tid < T) ssrc[tid] = w.src[w.n0 + tid];
-    if (gstage && w.gap)
-        for (int q = tid; q < T * Mg; q += nth) sgap[q] = w.gap[(long long)(w.n0 - q / Mg) * Mg + q % Mg];
+    if (gstage)  // rows n0 - T + 1 .. n0 are consecutive
+        for (int q = tid; q < T * Mg; q += nth) sgap[q] = w.gap[(long long)(w.n0 - T + 1) * Mg + q];
 
     // ---- load the region
     const bool cin = i0 >= 0 && i0 + VX <= P;           // the row pitch is a multiple of 32 words
@@ -502,7 +442,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
                             if (srcm >> (r * VX + v) & 1u) src = ssrc[t];
                         } else if (gapm >> (r * VX + v) & 1u) {
                             const int gi = (j0 + r - g.gy0) * g.gnx + (i0 + v - g.gx0);
-                            src = -c.eps_g * (gstage ? sgap[t * Mg + gi] : w.gap[(long long)(w.n0 - t) * Mg + gi]);
+                            src = -c.eps_g * (gstage ? sgap[(T - 1 - t) * Mg + gi] : w.gap[(long long)(w.n0 - t) * Mg + gi]);
                         }
                         x[r][v] = x[r][v] - src;
                     }
@@ -553,13 +493,13 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
 #pragma unroll
                     for (int r = 0; r < RPW; ++r)
 #pragma unroll
-                        for (int v = 0; v < VX; ++v) far |= Pair::far(em[r][v], term[r][v]);
+                        for (int v = 0; v < VX; ++v) far |= Pair::far(em[r][v], term[r][v] * Pair::SCALE);
                     if (__any_sync(0xffffffffu, far)) {
 #pragma unroll
                         for (int r = 0; r < RPW; ++r)
 #pragma unroll
                             for (int v = 0; v < VX; ++v)
-                                if (Pair::far(em[r][v], term[r][v])) {
+                                if (Pair::far(em[r][v], term[r][v] * Pair::SCALE)) {
                                     if (sens >> (r * VX + v) & 1u)
                                         w.G[d[r] + v] += (double)em[r][v] * (double)term[r][v];
                                     term[r][v] = R(0);
@@ -568,7 +508,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
 #pragma unroll
                     for (int r = 0; r < RPW; ++r)
 #pragma unroll
-                        for (int v = 0; v < VX; ++v) gp[r][v].add(em[r][v], term[r][v]);
+                        for (int v = 0; v < VX; ++v) gp[r][v].add(em[r][v], term[r][v] * Pair::SCALE);
                 }
             }
 #pragma unroll
@@ -626,7 +566,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
                 for (int v = 0; v < VX; ++v) {
                     if (!(sens >> (r * VX + v) & 1u)) continue;
                     if constexpr (F64) w.G[d[r] + v] = G[r][v];
-                    else w.G[d[r] + v] += (double)gp[r][v].hi + (double)gp[r][v].lo;
+                    else w.G[d[r] + v] += gp[r][v].value();
                 }
             }
         }
@@ -689,33 +629,14 @@ __global__ void k_rt2d_coef(const __grid_constant__ Geo2D g, int slot, const R *
 
 }  // namespace
 
-// Halo and tile rows for an nx x ny grid on `sms` SMs and at most `steps`
-// steps per launch: the least time per step, where a wave of blocks costs a
-// fixed part (launch, load, store: about 3 us) plus, per step, its rows that
-// are still needed (th + H - 1 on average), one row step being 0.026 us in
-// FP32 (two columns per lane) and 0.26 us in FP64.
+// A launch's fixed part is about 3 us; a row step is 0.025 us in FP32 (two
+// columns per lane) and 0.24 us in FP64.
 template <typename R>
 Rt2DPlan rt2d_plan(int nx, int ny, int sms, int steps)
 {
     using D = Shape<R>;
     constexpr bool F64 = sizeof(R) == 8;
-    constexpr double FIXED = F64 ? 10.0 : 130.0;
-    Rt2DPlan best{};
-    double cost = 0.0;
-    // FP32 tiles start on even columns, whatever the halo
-    for (int H = 4; H <= (!F64 && steps > 4 ? RT2D_MAX : 4); H += 2) {
-        const int tw = D::W - 2 * H, bx = (nx + tw - 1) / tw;
-        for (int nw = (2 * H + 2) / D::RPW; nw <= D::MAXW; ++nw) {
-            const int th = nw * D::RPW - 2 * H, by = (ny + th - 1) / th;
-            const long long waves = ((long long)bx * by + sms - 1) / sms;
-            const double k = (double)waves * (FIXED / H + th + H + 1);
-            if (best.halo == 0 || k < cost) {
-                cost = k;
-                best = Rt2DPlan{H, tw, th, nw, bx, by, 1};
-            }
-        }
-    }
-    return best;
+    return rt_tile_plan(nx, ny, sms, D::W, D::RPW, D::MAXW, !F64 && steps > 4 ? RT2D_MAX : 4, F64 ? 10.0 : 130.0);
 }
 
 template <typename R>

@@ -67,6 +67,55 @@ def test_blocked_equals_one_launch_per_step(real, kw):
     assert np.linalg.norm(g - g1) <= 1e-12 * np.linalg.norm(g1)
 
 
+def plane(nx, ny, real, **kw):
+    n = kw.pop("npml", 6)
+    d = kw.pop("design", (max(3, nx - 2 * n - 7), max(3, ny - 2 * n - 7)))
+    w = I.workload_2d_inplane(nx, ny, dx=20e-9, nsteps=kw.pop("nsteps", 170), npml=n, design=d, gap=kw.pop("gap", (2, 1)),
+                              real=real, material=I.SILVER, src_offset=kw.pop("src_offset", 1), **kw)
+    w.update(I.pulse(800e-9, 1200e12))
+    return w
+
+
+PLANE = [
+    ("f64", dict(nx=24, ny=25)), ("f64", dict(nx=49, ny=17, npml=3)), ("f64", dict(nx=57, ny=48, npml=0, src_offset=3)),
+    ("f64", dict(nx=7, ny=7, npml=1, design=(2, 2), gap=(1, 1), src_offset=1)),
+    ("f64", dict(nx=75, ny=70, snapshot_every=7)),
+    ("f32", dict(nx=41, ny=37)), ("f32", dict(nx=48, ny=33, snapshot_every=33)), ("f32", dict(nx=97, ny=95, npml=0)),
+    ("f32", dict(nx=130, ny=121, npml=10, gap=(24, 22), snapshot_every=45, nsteps=230)),
+    ("f32", dict(nx=321, ny=60, design=(280, 41), src_offset=0)),
+    ("f32", dict(nx=60, ny=61, npml=0, design=(59, 60), src_offset=10)),
+]
+
+
+@pytest.mark.parametrize("real,kw", PLANE)
+def test_inplane_blocked_equals_one_launch_per_half_step(real, kw):
+    """E in plane: the default (blocked launches, sensitivities summed from
+    the records of up to 32 adjoint steps) against one launch per half step,
+    with a gap record beyond the staging buffer, chunks of every length and
+    a design box up to the walls."""
+    w = plane(real=real, **kw)
+    rho = 0.1 * I.rho_uniform(w, 73)
+    W1, g1, h1, n1 = run(w, rho, 1)
+    W, g, h, n = run(w, rho, 0)
+    assert n < n1
+    assert np.isfinite(W1) and W1 > 0
+    assert W == W1
+    np.testing.assert_array_equal(h, h1)
+    assert np.linalg.norm(g - g1) <= 1e-12 * np.linalg.norm(g1)
+
+
+def test_inplane_blocked_with_kappa():
+    """kappa above 1 in the CPML: the product by 1/kappa and the sum with psi
+    may be rounded together, so FP64 agreement rather than equal bits."""
+    w = plane(60, 57, "f64", pml_kappa_max=3.0, pml_alpha_max=1e3)
+    rho = 0.1 * I.rho_uniform(w, 74)
+    W1, g1, h1, _ = run(w, rho, 1)
+    W, g, h, _ = run(w, rho, 0)
+    assert abs(W - W1) <= 1e-11 * W1
+    assert np.max(np.abs(h - h1)) <= 1e-11 * np.max(np.abs(h1))
+    assert np.linalg.norm(g - g1) <= 1e-11 * np.linalg.norm(g1)
+
+
 @pytest.mark.parametrize("amp", [1e-17, 1e16])
 def test_sensitivity_sum_follows_the_source_amplitude(amp):
     """The fields scale with src_amp, the gradient with its square: products
