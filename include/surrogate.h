@@ -49,6 +49,18 @@ int nn_im2col3(const float *x, int C, int B, int H, int W, float *col, void *str
 /* dx += the adjoint of nn_im2col3 applied to dcol. */
 int nn_col2im3_add(const float *dcol, int C, int B, int H, int W, float *dx, void *stream);
 
+/* 3 x 3 convolutions (stride 1, padding 1) with BF16 products, without im2col
+ * matrices.  Same results, bit for bit, as nn_im2col3 + nn_gemm_bf16
+ * (alpha = 1, beta = 0, the same scratch) + nn_bias_act / nn_col2im3_add.
+ * nn_conv3_fwd: y = act(w * x + bias), x [ci][B][H][W], w [co][ci 9], y
+ * [co][B][H][W].  nn_conv3_dgrad: dx = (add: +=) the input gradient.
+ * nn_conv3_wgrad: gw = the weight gradient. */
+int nn_conv3_fwd(const float *x, const float *w, const float *bias, float *y, int ci, int co, int B, int H, int W,
+                 int relu, float *work, long long work_elems, void *stream);
+int nn_conv3_dgrad(const float *dy, const float *w, float *dx, int ci, int co, int B, int H, int W, int add, void *stream);
+int nn_conv3_wgrad(const float *dy, const float *x, float *gw, int ci, int co, int B, int H, int W, float *work,
+                   long long work_elems, void *stream);
+
 /* y[c][p] = act(y[c][p] + bias[c]) for c < Cout, p < P; act = ReLU if relu. */
 int nn_bias_act(float *y, const float *bias, int Cout, long long P, int relu, void *stream);
 

@@ -414,6 +414,16 @@ static int splitk(int M, int N, int K, long long tiles, int step, long long work
     return (K + *kc - 1) / *kc;
 }
 
+// The K slices nn_gemm_bf16 takes for an M x N x K product, for the kernels
+// that reproduce its sums (conv.cu).
+int nn_splitk_bf16(int M, long long N, long long K, long long work_elems, long long *kc)
+{
+    int k = 0;
+    const int s = splitk(M, (int)N, (int)K, (N + BN - 1) / BN * ((M + BM - 1) / BM), BK, work_elems, &k);
+    *kc = k;
+    return s;
+}
+
 int nn_gemm(int transA, int transB, int M, int N, int K, float alpha, const float *A, int lda, const float *B, int ldb,
             float beta, float *C, int ldc, float *work, long long work_elems, void *stream)
 {

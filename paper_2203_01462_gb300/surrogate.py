@@ -37,6 +37,12 @@ _FNS = {
     "nn_adam": [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_longlong, C.c_float, C.c_float, C.c_float,
                 C.c_float, C.c_int, C.c_void_p],
     "nn_zero": [C.c_void_p, C.c_longlong, C.c_void_p],
+    "nn_conv3_fwd": [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
+                     C.c_int, C.c_void_p, C.c_longlong, C.c_void_p],
+    "nn_conv3_dgrad": [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
+                       C.c_void_p],
+    "nn_conv3_wgrad": [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p,
+                       C.c_longlong, C.c_void_p],
     "nn_gemm_bf16": [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_float, C.c_void_p, C.c_int, C.c_void_p,
                      C.c_int, C.c_float, C.c_void_p, C.c_int, C.c_void_p, C.c_longlong, C.c_void_p],
 }
@@ -105,8 +111,9 @@ class UNet:
         self.skip = {"enc1b": ("cat1", 2 * b, b), "enc2b": ("cat2", 4 * b, 2 * b), "enc3b": ("cat3", 8 * b, 4 * b)}
         col_elems = max(ci * k * k * B * sz[self._level(n)][0] * sz[self._level(n)][1]
                         for n, ci, co, k in self.layers)
-        self.col = torch.zeros(col_elems, **f32)
-        self.dcol = torch.zeros(col_elems, **f32)
+        if precision == "f32":  # im2col scratch; the BF16 convolutions gather their operands themselves
+            self.col = torch.zeros(col_elems, **f32)
+            self.dcol = torch.zeros(col_elems, **f32)
         # split-K scratch of the GEMMs (partial products summed in a fixed
         # order): room for 16 slices of the largest weight matrix
         self.gemm_work = torch.zeros(max(1 << 20, 16 * max(co * ci * k * k for n, ci, co, k in self.layers)), **f32)
@@ -160,6 +167,10 @@ class UNet:
     def _conv_fwd(self, name, ci, co, k, x, y, relu):
         L, st = _nn(), self._st()
         Bhw = x[0].numel()
+        if k == 3 and self.precision == "bf16":
+            _ck(L.nn_conv3_fwd(_p(x), _p(self.w[name]), _p(self.b[name]), _p(y), ci, co, self.B, x.shape[2], x.shape[3],
+                               int(relu), _p(self.gemm_work), self.gemm_work.numel(), st), "conv fwd")
+            return
         if k == 3:
             _ck(L.nn_im2col3(_p(x), ci, self.B, x.shape[2], x.shape[3], _p(self.col), st), "im2col")
             src = self.col
@@ -173,6 +184,13 @@ class UNet:
         L, st = _nn(), self._st()
         Bhw = x[0].numel()
         _ck(L.nn_act_bwd_bias(_p(y), _p(dy), _p(self.gb[name]), co, Bhw, int(relu), st), "act_bwd")
+        if k == 3 and self.precision == "bf16":
+            _ck(L.nn_conv3_wgrad(_p(dy), _p(x), _p(self.gw[name]), ci, co, self.B, x.shape[2], x.shape[3],
+                                 _p(self.gemm_work), self.gemm_work.numel(), st), "conv wgrad")
+            if dx is not None:
+                _ck(L.nn_conv3_dgrad(_p(dy), _p(self.w[name]), _p(dx), ci, co, self.B, x.shape[2], x.shape[3], 0, st),
+                    "conv dgrad")
+            return
         if k == 3:
             _ck(L.nn_im2col3(_p(x), ci, self.B, x.shape[2], x.shape[3], _p(self.col), st), "im2col")
             src = self.col
@@ -214,8 +232,10 @@ class UNet:
     def backward(self, dout: torch.Tensor) -> None:
         """dout: dL/d(output) [1][B][H][W]; fills the parameter gradients."""
         L, st, a, g, b = _nn(), self._st(), self.a, self.g, self.base
-        for t in g.values():
-            _ck(L.nn_zero(_p(t), t.numel(), st), "zero")
+        # gradients that are added to before anything is stored in them (the BF16
+        # convolutions store the first term of the others)
+        for k in ("botb", "dec3b", "dec2b", "dec1b") if self.precision == "bf16" else g:
+            _ck(L.nn_zero(_p(g[k]), g[k].numel(), st), "zero")
         g["head"].copy_(dout)
         pools = {"enc1b": "p1", "enc2b": "p2", "enc3b": "p3"}
         ups = {"botb": ("cat3", 8 * b), "dec3b": ("cat2", 4 * b), "dec2b": ("cat1", 2 * b)}
