@@ -81,6 +81,9 @@ int nn_mse(const float *y, const float *t, long long n, float *dy, double *loss,
 /* Adam step `step` (>= 1) on n parameters: m, v are the moment buffers. */
 int nn_adam(float *p, const float *g, float *m, float *v, long long n, float lr, float beta1, float beta2, float eps,
             int step, void *stream);
+/* The same on `count` tensors (host arrays of device pointers and sizes), 64 per launch. */
+int nn_adam_multi(int count, float *const *p, const float *const *g, float *const *m, float *const *v, const long long *n,
+                  float lr, float beta1, float beta2, float eps, int step, void *stream);
 
 /* x[0 .. n) = 0. */
 int nn_zero(float *x, long long n, void *stream);

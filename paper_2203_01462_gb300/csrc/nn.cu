@@ -8,6 +8,7 @@
 // W[Cout][Cin K K] . col[Cin K K][B H W], and concatenating along channels is
 // placing tensors next to each other in memory.
 #include <cuda_bf16.h>
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -203,6 +204,52 @@ __global__ void __launch_bounds__(1024) k_relu_bwd_bias(const float *y, float *d
     }
 }
 
+// The same for long rows: the 32 warps of a channel's block as a cluster of
+// eight blocks.  One block per channel left 24 of 152 SMs busy on the widest
+// layers (82 us for 24 x 524288 values, 150 MB; 26 us so).  Every thread adds
+// the values it would have added there, in that order, and the warps' sums
+// are added in theirs: the same bits.
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(128)
+k_relu_bwd_bias8(const float *__restrict__ y, float *dy, float *db, long long P, int relu)
+{
+    __shared__ float part[32];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = blockIdx.x & 7, c = blockIdx.x >> 3, warp = rank * 4 + (threadIdx.x >> 5);
+    const float4 *y4 = reinterpret_cast<const float4 *>(y + (long long)c * P);
+    float4 *d4 = reinterpret_cast<float4 *>(dy + (long long)c * P);
+    float s = 0.0f;
+    for (long long p0 = rank * 128 + threadIdx.x; p0 < P / 4; p0 += 8 * 1024) {
+        float4 g[8], v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (p0 + q * 1024 < P / 4) {
+                g[q] = d4[p0 + q * 1024];
+                if (relu) v[q] = y4[p0 + q * 1024];
+            }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (p0 + q * 1024 < P / 4) {
+                if (relu) {
+                    if (!(v[q].x > 0.0f)) g[q].x = 0.0f;
+                    if (!(v[q].y > 0.0f)) g[q].y = 0.0f;
+                    if (!(v[q].z > 0.0f)) g[q].z = 0.0f;
+                    if (!(v[q].w > 0.0f)) g[q].w = 0.0f;
+                    d4[p0 + q * 1024] = g[q];
+                }
+                s += (g[q].x + g[q].y) + (g[q].z + g[q].w);
+            }
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) *cl.map_shared_rank(part + warp, 0) = s;
+    cl.sync();
+    if (rank == 0 && threadIdx.x < 32) {
+        s = part[threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) db[c] = s;
+    }
+}
+
 // 2 x 2 average pooling of planes [n][H][W] -> [n][H/2][W/2] and its adjoint.
 __global__ void k_pool2(const float *x, long long planes, int H, int W, float *y)
 {
@@ -250,6 +297,71 @@ __global__ void k_up2_bwd(const float *dy, long long planes, int h, int w, float
     }
 }
 
+// The resampling passes with rows of even w and 16-byte aligned planes: a
+// thread has two coarse pixels, a float2, and their 2 x 2 fine ones, two
+// float4 (the passes are bound by HBM: one value per thread with its index
+// divisions took 99 us instead of 19 for k_up2 to 48 x 8 planes of 256^2, 55
+// instead of 15 for k_pool2_bwd).  F(coarse, fine, w4) on float2 / float4
+// words: fine[0] and fine[w4] are the two rows.
+template <class F>
+__device__ __forceinline__ void each_pair(long long planes, int h, int w, F f)
+{
+    const int w2 = w / 2;
+    const long long n = planes * h * w2;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
+        f(e, (e / w2 * 2) * w2 + e % w2, w2);  // fine rows of w2 float4
+}
+
+__global__ void k_pool2_v(const float4 *__restrict__ x, long long planes, int h, int w, float2 *y)
+{
+    each_pair(planes, h, w, [&](long long c, long long f, int w4) {
+        const float4 a = x[f], b = x[f + w4];
+        y[c] = make_float2(0.25f * (a.x + a.y + b.x + b.y), 0.25f * (a.z + a.w + b.z + b.w));
+    });
+}
+
+__global__ void k_pool2_bwd_v(const float2 *__restrict__ dy, long long planes, int h, int w, float4 *dx)
+{
+    each_pair(planes, h, w, [&](long long c, long long f, int w4) {
+        const float2 g = dy[c];
+        float4 a = dx[f], b = dx[f + w4];
+        a.x += 0.25f * g.x;
+        a.y += 0.25f * g.x;
+        a.z += 0.25f * g.y;
+        a.w += 0.25f * g.y;
+        b.x += 0.25f * g.x;
+        b.y += 0.25f * g.x;
+        b.z += 0.25f * g.y;
+        b.w += 0.25f * g.y;
+        dx[f] = a;
+        dx[f + w4] = b;
+    });
+}
+
+__global__ void k_up2_v(const float2 *__restrict__ x, long long planes, int h, int w, float4 *y)
+{
+    each_pair(planes, h, w, [&](long long c, long long f, int w4) {
+        const float2 v = x[c];
+        y[f] = y[f + w4] = make_float4(v.x, v.x, v.y, v.y);
+    });
+}
+
+__global__ void k_up2_bwd_v(const float4 *__restrict__ dy, long long planes, int h, int w, float2 *dx)
+{
+    each_pair(planes, h, w, [&](long long c, long long f, int w4) {
+        const float4 a = dy[f], b = dy[f + w4];
+        float2 v = dx[c];
+        v.x += a.x + a.y + b.x + b.y;
+        v.y += a.z + a.w + b.z + b.w;
+        dx[c] = v;
+    });
+}
+
+bool pairs_ok(int w, const void *coarse, const void *fine)
+{
+    return w % 2 == 0 && ((uintptr_t)coarse & 7) == 0 && ((uintptr_t)fine & 15) == 0;
+}
+
 // loss = mean (y - t)^2 (FP64 accumulation into *loss, which must start at 0);
 // dy = 2 (y - t) / n.
 __global__ void k_mse(const float *y, const float *t, long long n, float *dy, double *loss)
@@ -265,17 +377,43 @@ __global__ void k_mse(const float *y, const float *t, long long n, float *dy, do
     if ((threadIdx.x & 31) == 0) atomicAdd(loss, s / (double)n);
 }
 
-__global__ void k_adam(float *p, const float *g, float *m, float *v, long long n, float lr, float b1, float b2,
-                       float eps, float c1, float c2)
+// Adam on up to ADAM_T tensors in one launch: blocks of ADAM_E elements, the
+// blocks of tensor i from first[i] on.  The base-24 network's 30 tensors took
+// 30 launches of 4 us each, most of them a few blocks; 11 us so.
+constexpr int ADAM_T = 64, ADAM_E = 1024;
+
+struct AdamList {
+    float *p[ADAM_T], *m[ADAM_T], *v[ADAM_T];
+    const float *g[ADAM_T];
+    long long n[ADAM_T];
+    int first[ADAM_T + 1];
+    int count;
+};
+
+__global__ void __launch_bounds__(TPB) k_adam(const __grid_constant__ AdamList L, float lr, float b1, float b2, float eps,
+                                              float c1, float c2)
 {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const float gg = g[e];
-        const float mm = b1 * m[e] + (1.0f - b1) * gg;
-        const float vv = b2 * v[e] + (1.0f - b2) * gg * gg;
-        m[e] = mm;
-        v[e] = vv;
-        p[e] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+    int i = 0, hi = L.count - 1;
+    while (i < hi) {
+        const int mid = (i + hi + 1) / 2;
+        if (L.first[mid] <= (int)blockIdx.x) i = mid;
+        else hi = mid - 1;
     }
+    float *p = L.p[i], *m = L.m[i], *v = L.v[i];
+    const float *g = L.g[i];
+    const long long n = L.n[i], step = (long long)(L.first[i + 1] - L.first[i]) * ADAM_E;
+    for (long long e0 = (long long)(blockIdx.x - L.first[i]) * ADAM_E; e0 < n; e0 += step)
+#pragma unroll
+        for (int q = 0; q < ADAM_E / TPB; ++q) {
+            const long long e = e0 + q * TPB + threadIdx.x;
+            if (e >= n) break;
+            const float gg = g[e];
+            const float mm = b1 * m[e] + (1.0f - b1) * gg;
+            const float vv = b2 * v[e] + (1.0f - b2) * gg * gg;
+            m[e] = mm;
+            v[e] = vv;
+            p[e] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+        }
 }
 
 __global__ void k_zero_f(float *x, long long n)
@@ -490,7 +628,10 @@ int nn_act_bwd_bias(const float *y, float *dy, float *db, int Cout, long long P,
     if (!y || !dy || !db || Cout <= 0 || P <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     const int vec = (P & 3) == 0 && (((uintptr_t)y | (uintptr_t)dy) & 15) == 0;
-    k_relu_bwd_bias<<<Cout, 1024, 0, st>>>(y, dy, db, P, relu, vec);
+    if (vec && P >= 8 * 4096)  // eight values' loads in flight per thread; below, one block has them all at once
+        k_relu_bwd_bias8<<<8 * Cout, 128, 0, st>>>(y, dy, db, P, relu);
+    else
+        k_relu_bwd_bias<<<Cout, 1024, 0, st>>>(y, dy, db, P, relu, vec);
     return status(st);
 }
 
@@ -498,7 +639,10 @@ int nn_pool2(const float *x, long long planes, int H, int W, float *y, void *str
 {
     if (!x || !y || planes <= 0 || H < 2 || W < 2 || (H | W) & 1) return 1;
     cudaStream_t st = (cudaStream_t)stream;
-    k_pool2<<<blocks_for(planes * (H / 2) * (W / 2)), TPB, 0, st>>>(x, planes, H, W, y);
+    if (pairs_ok(W / 2, y, x))
+        k_pool2_v<<<blocks_for(planes * (H / 2) * (W / 4)), TPB, 0, st>>>((const float4 *)x, planes, H / 2, W / 2, (float2 *)y);
+    else
+        k_pool2<<<blocks_for(planes * (H / 2) * (W / 2)), TPB, 0, st>>>(x, planes, H, W, y);
     return status(st);
 }
 
@@ -506,7 +650,10 @@ int nn_pool2_bwd_add(const float *dy, long long planes, int H, int W, float *dx,
 {
     if (!dy || !dx || planes <= 0 || H < 2 || W < 2 || (H | W) & 1) return 1;
     cudaStream_t st = (cudaStream_t)stream;
-    k_pool2_bwd<<<blocks_for(planes * H * W), TPB, 0, st>>>(dy, planes, H, W, dx);
+    if (pairs_ok(W / 2, dy, dx))
+        k_pool2_bwd_v<<<blocks_for(planes * (H / 2) * (W / 4)), TPB, 0, st>>>((const float2 *)dy, planes, H / 2, W / 2, (float4 *)dx);
+    else
+        k_pool2_bwd<<<blocks_for(planes * H * W), TPB, 0, st>>>(dy, planes, H, W, dx);
     return status(st);
 }
 
@@ -514,7 +661,10 @@ int nn_up2(const float *x, long long planes, int h, int w, float *y, void *strea
 {
     if (!x || !y || planes <= 0 || h <= 0 || w <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
-    k_up2<<<blocks_for(planes * 4 * h * w), TPB, 0, st>>>(x, planes, h, w, y);
+    if (pairs_ok(w, x, y))
+        k_up2_v<<<blocks_for(planes * h * (w / 2)), TPB, 0, st>>>((const float2 *)x, planes, h, w, (float4 *)y);
+    else
+        k_up2<<<blocks_for(planes * 4 * h * w), TPB, 0, st>>>(x, planes, h, w, y);
     return status(st);
 }
 
@@ -522,7 +672,10 @@ int nn_up2_bwd_add(const float *dy, long long planes, int h, int w, float *dx, v
 {
     if (!dy || !dx || planes <= 0 || h <= 0 || w <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
-    k_up2_bwd<<<blocks_for(planes * h * w), TPB, 0, st>>>(dy, planes, h, w, dx);
+    if (pairs_ok(w, dx, dy))
+        k_up2_bwd_v<<<blocks_for(planes * h * (w / 2)), TPB, 0, st>>>((const float4 *)dy, planes, h, w, (float2 *)dx);
+    else
+        k_up2_bwd<<<blocks_for(planes * h * w), TPB, 0, st>>>(dy, planes, h, w, dx);
     return status(st);
 }
 
@@ -535,14 +688,38 @@ int nn_mse(const float *y, const float *t, long long n, float *dy, double *loss,
     return status(st);
 }
 
+int nn_adam_multi(int count, float *const *p, const float *const *g, float *const *m, float *const *v, const long long *n,
+                  float lr, float beta1, float beta2, float eps, int step, void *stream)
+{
+    if (count <= 0 || !p || !g || !m || !v || !n || step < 1) return 1;
+    for (int i = 0; i < count; ++i)
+        if (!p[i] || !g[i] || !m[i] || !v[i] || n[i] <= 0) return 1;
+    cudaStream_t st = (cudaStream_t)stream;
+    const float c1 = 1.0f - powf(beta1, (float)step), c2 = 1.0f - powf(beta2, (float)step);
+    for (int i0 = 0; i0 < count; i0 += ADAM_T) {
+        AdamList L;
+        L.count = count - i0 < ADAM_T ? count - i0 : ADAM_T;
+        int blocks = 0;
+        for (int i = 0; i < L.count; ++i) {
+            L.p[i] = p[i0 + i];
+            L.g[i] = g[i0 + i];
+            L.m[i] = m[i0 + i];
+            L.v[i] = v[i0 + i];
+            L.n[i] = n[i0 + i];
+            L.first[i] = blocks;
+            const long long b = (L.n[i] + ADAM_E - 1) / ADAM_E;
+            blocks += (int)(b < 152 * 16 ? b : 152 * 16);
+        }
+        L.first[L.count] = blocks;
+        k_adam<<<blocks, TPB, 0, st>>>(L, lr, beta1, beta2, eps, c1, c2);
+    }
+    return status(st);
+}
+
 int nn_adam(float *p, const float *g, float *m, float *v, long long n, float lr, float beta1, float beta2, float eps,
             int step, void *stream)
 {
-    if (!p || !g || !m || !v || n <= 0 || step < 1) return 1;
-    cudaStream_t st = (cudaStream_t)stream;
-    const float c1 = 1.0f - powf(beta1, (float)step), c2 = 1.0f - powf(beta2, (float)step);
-    k_adam<<<blocks_for(n), TPB, 0, st>>>(p, g, m, v, n, lr, beta1, beta2, eps, c1, c2);
-    return status(st);
+    return nn_adam_multi(1, &p, &g, &m, &v, &n, lr, beta1, beta2, eps, step, stream);
 }
 
 int nn_zero(float *x, long long n, void *stream)

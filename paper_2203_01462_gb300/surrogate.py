@@ -36,6 +36,8 @@ _FNS = {
     "nn_mse": [C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p, C.c_void_p, C.c_void_p],
     "nn_adam": [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_longlong, C.c_float, C.c_float, C.c_float,
                 C.c_float, C.c_int, C.c_void_p],
+    "nn_adam_multi": [C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_float, C.c_float,
+                      C.c_float, C.c_float, C.c_int, C.c_void_p],
     "nn_zero": [C.c_void_p, C.c_longlong, C.c_void_p],
     "nn_conv3_fwd": [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
                      C.c_int, C.c_void_p, C.c_longlong, C.c_void_p],
@@ -260,10 +262,12 @@ class UNet:
         d = dout.clone()
         self.backward(d)
         self.step += 1
-        for key, t in self._params():
-            grad = self.gw[key[:-2]] if key.endswith(".w") else self.gb[key[:-2]]
-            _ck(L.nn_adam(_p(t), _p(grad), _p(self.m[key]), _p(self.v[key]), t.numel(), lr, 0.9, 0.999, 1e-8,
-                          self.step, st), "adam")
+        ps = list(self._params())
+        gs = [self.gw[k[:-2]] if k.endswith(".w") else self.gb[k[:-2]] for k, _ in ps]
+        ptrs = [(C.c_void_p * len(ps))(*[t.data_ptr() for t in ts])
+                for ts in ([t for _, t in ps], gs, [self.m[k] for k, _ in ps], [self.v[k] for k, _ in ps])]
+        sizes = (C.c_longlong * len(ps))(*[t.numel() for _, t in ps])
+        _ck(L.nn_adam_multi(len(ps), *ptrs, sizes, lr, 0.9, 0.999, 1e-8, self.step, st), "adam")
         return self.loss
 
     def grads(self) -> dict:
