@@ -67,9 +67,9 @@ def workload(name: str, nsteps: int | None):
 
 
 # DRAM bytes (read + write) of the forward step kernels of one time step,
-# measured by ncu on each workload's own grid (k_step2d<float,0>; k_h3d +
+# measured by ncu on each workload's own grid (k_rt2d<float,0>, 6 steps per launch; k_h3d +
 # k_e3d<float,0>); entries are removed whenever a kernel changes.
-NCU_TRAFFIC_PER_STEP = {"cfg_2d_2048": 74.2e6, "cfg_3d_256": 1298.4e6}
+NCU_TRAFFIC_PER_STEP = {"cfg_2d_2048": 14.5e6, "cfg_3d_256": 1298.4e6}
 
 
 def damping(k: int) -> float:
@@ -356,11 +356,6 @@ def main() -> None:
     dev = torch.device("cuda", local)
     stream = torch.cuda.Stream(dev)
     s = Solver(w, device=dev, stream=stream)
-    # 2D E_z workloads: keep 30 % of the ping-pong state persisting in L2
-    # (the share that measured fastest; results are bit-identical)
-    l2_share = 0.3 if (w["ndim"] == 2 and not I.inplane(w)) else 0.0
-    if l2_share:
-        s.set_l2_residency(l2_share)
     rho = torch.tensor(I.rho_uniform(w, rank), dtype=torch.float32 if w["real"] == "f32" else torch.float64,
                        device=dev)
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
@@ -463,13 +458,12 @@ def main() -> None:
         config=dict(workload=I.describe(w), grid=I.grid_shape(w), nsteps=N, design=list(I.design_shape(w))[::-1],
                     snapshot_every=w["snapshot_every"], snapshot_dtype=w.get("snapshot_dtype", "f32"),
                     parallelism="replicas" if world > 1 else "1 GPU",
-                    l2="flushed (256 MB write) between timed steps",
-                    l2_residency=l2_share),
+                    l2="flushed (256 MB write) between timed steps"),
         roofline=dict(bound="hbm", achieved=achieved, peak=hbm, unit="GB/s", frac=achieved / hbm,
                       traffic=NCU_TRAFFIC_PER_STEP.get(w["name"]), traffic_unit="bytes per forward step",
                       algorithmic_bytes_per_step=ab["forward"],
-                      kernel=("k_hp + k_ep<float,0> (forward H and E half steps, E in plane)" if I.inplane(w)
-                              else "k_step2d<float,0> (fused forward leapfrog step)") if w["ndim"] == 2
+                      kernel=("k_rt2dp<float,0> (blocked forward leapfrog steps, E in plane)" if I.inplane(w)
+                              else "k_rt2d<float,0> (blocked forward leapfrog steps)") if w["ndim"] == 2
                       else "k_h3d + k_e3d<float,0> (forward H and E half steps; a plane wave's face corrections "
                       "inside them)",
                       peak_source=peak_src),

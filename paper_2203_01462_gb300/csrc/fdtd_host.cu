@@ -673,11 +673,12 @@ struct Ctx2D final : fdtd_ctx {
             // Measured, launch per step against blocked (us per forward /
             // full-history adjoint step): FP32 316^2 6.9 / 7.5 against 1.02 /
             // 1.28, 500^2 7.5 / 7.6 against 2.1 / 2.3, 1000^2 10.6 / 10.4
-            // against 5.7 / 6.5, 1400^2 13.1 / 15.3 against 10.1 / 11.6, 2048^2
-            // 23.8 / 27.7 against 21.7 / 24.7 (but 21.2 with the L2 window,
-            // which the blocked launches do not take); FP64 160^2 12.1 / 15.1
-            // against 3.3 / 3.3, 1000^2 52 / 72 against 49 / 53.
-            rt_auto = ncells <= (sizeof(R) == 4 ? 1LL << 21 : 1LL << 20);
+            // against 4.9 / 6.2, 1400^2 13.1 / 15.3 against 8.0 / 10.4, 2048^2
+            // 23.2 / 25 against 17.3 / 22 (21.2 forward with the L2 window,
+            // which the blocked launches do not take), 4096^2 77 / 86 against
+            // 69 / 86; FP64 160^2 12.1 / 15.1 against 3.3 / 3.3, 1000^2 52 /
+            // 72 against 49 / 53.
+            rt_auto = sizeof(R) == 4 || ncells <= 1LL << 20;
         }
         return cuda_ok(cudaStreamSynchronize(st));
     }

@@ -90,11 +90,11 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
     const Coef<R> &c = coef_at<R>(slot);
     const int lane = threadIdx.x, wi = threadIdx.y, nw = blockDim.y, tid = wi * 32 + lane, nth = nw * 32;
     const int T = w.count, H = w.halo, nx = g.nx, ny = g.ny, np = g.npml, P = g.px, np2 = 2 * np;
-    const int xr = blockIdx.x * w.tw - H, yr = blockIdx.y * w.th - H;  // region origin (grid)
-    const int i0 = xr + lane * VX, j0 = yr + wi * RPW;                 // this thread's first node
     const int Mg = g.gnx * g.gny;
     const R S = c.S;
 
+    const int xr = blockIdx.x * w.tw - H, yr = blockIdx.y * w.th - H;  // region origin (grid)
+    const int i0 = xr + lane * VX, j0 = yr + wi * RPW;                 // this thread's first node
     R *sU = (R *)smem_raw;                 // [2][nw + 1][W]: a warp's first Ez row, read by the warp below
     R *sD = sU + 2 * (nw + 1) * W;         // [2][nw + 1][W]: a warp's last Ez row (FP64: last Hx row), read by the warp above
     R *xt = sD + 2 * (nw + 1) * W;         // [6][W]: bE cE kiE bH cH kiH of the columns
@@ -145,8 +145,19 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
     if (gstage)  // rows n0 - T + 1 .. n0 are consecutive
         for (int q = tid; q < T * Mg; q += nth) sgap[q] = w.gap[(long long)(w.n0 - T + 1) * Mg + q];
 
+    // Everything from the loads to the stores, one instance per kind of
+    // region.  V: every node is a plain one of the background; D: of the
+    // design box; both clear of walls, absorbing layer, gap and source.  On
+    // large grids nearly all regions are, and the tests for anything else were
+    // 600 of a launch's 1080 instructions per warp: 2048^2 22.5 -> 17.8 us per
+    // forward step, 27 -> 23.5 per adjoint step, 1000^2 5.9 -> 4.9.  (Copying
+    // the next tile's state into shared memory while one is stepped, in
+    // persistent blocks, gained nothing on top: 18.5; instruction issue, at
+    // half its rate, and the step's barrier are what is left.)
+    auto body = [&](auto vc, auto dc) {
+    constexpr bool V = decltype(vc)::value, D = decltype(dc)::value, PL = V || D;
     // ---- load the region
-    const bool cin = i0 >= 0 && i0 + VX <= P;           // the row pitch is a multiple of 32 words
+    const bool cin = PL || (i0 >= 0 && i0 + VX <= P);  // the row pitch is a multiple of 32 words
     const bool vdx = i0 >= g.dxa && i0 < g.dxa + g.dp;  // and the design box's columns start on a multiple of 4
     const bool own_x = lane * VX >= H && lane * VX < H + w.tw && i0 < nx;
     R ez[RPW][VX], hx[RPW][VX], hy[RPW][VX], jj[RPW][VX], ca[RPW][VX], cb[RPW][VX], bj[RPW][VX], hxd[VX];
@@ -162,7 +173,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
         zero(ca[r]); zero(cb[r]); zero(bj[r]); zero(a1[r]); zero(a2[r]);
         if (own_x && wi * RPW + r >= H && wi * RPW + r < H + w.th && j < ny) ownr |= 1u << r;
         d[r] = (long long)(j - g.dy0) * g.dp + (i0 - g.dxa);
-        if (vdx && in_range(j, g.dy0, g.dny)) {
+        if (D || (!V && vdx && in_range(j, g.dy0, g.dny))) {
             desr |= 1u << r;
             ldv(w.coef + d[r], ca[r]);
             ldv(w.coef + w.Mdi + d[r], cb[r]);
@@ -190,19 +201,19 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
             G[r][v] = 0.0;
             gp[r][v] = Pair{0.0f, 0.0f};
         }
-        if ((unsigned)j < (unsigned)ny && cin) {
+        if (PL || ((unsigned)j < (unsigned)ny && cin)) {
             const long long q = (long long)j * P + i0;
             ldv(in.Ez + q, ez[r]);
             ldv(in.Hx + q, hx[r]);
             ldv(in.Hy + q, hy[r]);
-            if (r == 0 && j >= 1 && !F64) ldv(in.Hx + q - P, hxd);
-            if (desr >> r & 1u) {
+            if (r == 0 && (PL || j >= 1) && !F64) ldv(in.Hx + q - P, hxd);
+            if (D || desr >> r & 1u) {
                 ldv(in.J + d[r], jj[r]);
                 if (MODE == 1 && F64 && (ownr >> r & 1u))
 #pragma unroll
                     for (int v = 0; v < VX; ++v) G[r][v] = w.G[d[r] + v];
             }
-            if (xp) {
+            if (!PL && xp) {
 #pragma unroll
                 for (int v = 0; v < VX; ++v) {
                     const int i = i0 + v;
@@ -212,7 +223,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
                     if (sh >= 0) phx[r][v] = in.phyx[(long long)j * np2 + sh];
                 }
             }
-            if (yp) {
+            if (!PL && yp) {
                 const int te = slab_e(j, ny, np), th = slab_h(j, ny, np);
                 if (te >= 0) ldv(in.pezy + (long long)te * P + i0, pey[r]);
                 if (th >= 0) ldv(in.phxy + (long long)th * P + i0, phy[r]);
@@ -227,31 +238,31 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
     // components whose half-step neighbour exists.
     R Sx[VX], Sy[RPW];
 #pragma unroll
-    for (int v = 0; v < VX; ++v) Sx[v] = (i0 + v >= 0 && i0 + v + 1 < nx) ? S : R(0);
+    for (int v = 0; v < VX; ++v) Sx[v] = PL || (i0 + v >= 0 && i0 + v + 1 < nx) ? S : R(0);
 #pragma unroll
     for (int r = 0; r < RPW; ++r) {
         const int j = j0 + r;
-        Sy[r] = (j >= 0 && j + 1 < ny) ? S : R(0);
+        Sy[r] = PL || (j >= 0 && j + 1 < ny) ? S : R(0);
 #pragma unroll
         for (int v = 0; v < VX; ++v) {
             const int i = i0 + v;
-            const bool upd = i >= 1 && i <= nx - 2 && j >= 1 && j <= ny - 2;
-            const bool gap = in_range(i, g.gx0, g.gnx) && in_range(j, g.gy0, g.gny);
+            const bool upd = PL || (i >= 1 && i <= nx - 2 && j >= 1 && j <= ny - 2);
+            const bool gap = !PL && in_range(i, g.gx0, g.gnx) && in_range(j, g.gy0, g.gny);
             if (bj[r][v] == R(0)) cb[r][v] = gap ? c.inv_eps_g : c.inv_eps_s;
             if (!upd) cb[r][v] = R(0);
             if (gap) gapm |= 1u << (r * VX + v);
-            if (MODE == 0 && in_range(i, g.sx0, g.sx1 - g.sx0) && in_range(j, g.sy0, g.sy1 - g.sy0))
+            if (!PL && MODE == 0 && in_range(i, g.sx0, g.sx1 - g.sx0) && in_range(j, g.sy0, g.sy1 - g.sy0))
                 srcm |= 1u << (r * VX + v);
         }
     }
-    const R Syd = (j0 - 1 >= 0 && j0 < ny) ? S : R(0);
+    const R Syd = PL || (j0 - 1 >= 0 && j0 < ny) ? S : R(0);
     // FORM 1: nodes of the step kernel's plain vector tiles take its S / eps
     // as one factor of the unscaled curl (different bits in the denormal
     // range only, but rounding noise there outlives the front it starts in).
     R Sc = S;
-    if (FORM == 1) {
+    if (FORM == 1 && !D) {
         const int tx0 = i0 & ~(STEP2D_TX - 1), ty0 = j0 & ~(STEP2D_TY - 1);
-        if (i0 >= 0 && j0 >= 0 && step2d_vector_tile(nx, ny, np, tx0, ty0) && !step2d_touches(g, MODE, tx0, ty0)) {
+        if ((PL || (i0 >= 0 && j0 >= 0)) && step2d_vector_tile(nx, ny, np, tx0, ty0) && !step2d_touches(g, MODE, tx0, ty0)) {
             Sc = R(1);
 #pragma unroll
             for (int r = 0; r < RPW; ++r)
@@ -263,7 +274,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
     // lie in the rows' absorbing layer; it holds nodes with a source term,
     // own gap nodes to record.
     bool yph = false, ype = false;
-    if (yp) {
+    if (!PL && yp) {
 #pragma unroll
         for (int r = -1; r < RPW; ++r) {
             const int j = j0 + r;
@@ -273,8 +284,8 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
             }
         }
     }
-    const bool anysrc = __any_sync(0xffffffffu, (MODE == 0 ? srcm : gapm) != 0);
-    const bool anygap = MODE == 0 && w.gap && __any_sync(0xffffffffu, gapm != 0 && ownr != 0);
+    const bool anysrc = !PL && __any_sync(0xffffffffu, (MODE == 0 ? srcm : gapm) != 0);
+    const bool anygap = !PL && MODE == 0 && w.gap && __any_sync(0xffffffffu, gapm != 0 && ownr != 0);
     // Block-uniform: the region holds design columns.
     const bool dru = xr < g.dxa + g.dp && xr + W > g.dxa && yr < g.dy0 + g.dny && yr + nw * RPW > g.dy0;
     // Warp-uniform: it holds own rows; own Drude nodes (node bits).
@@ -298,10 +309,10 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
     R tx[4][VX];  // CPML b, c of this thread's columns (E, then H); 1/kappa stays in shared memory
 #pragma unroll
     for (int v = 0; v < VX; ++v) {
-        tx[0][v] = xp ? xt[lane * VX + v] : R(0);
-        tx[1][v] = xp ? xt[W + lane * VX + v] : R(0);
-        tx[2][v] = xp ? xt[3 * W + lane * VX + v] : R(0);
-        tx[3][v] = xp ? xt[4 * W + lane * VX + v] : R(0);
+        tx[0][v] = !PL && xp ? xt[lane * VX + v] : R(0);
+        tx[1][v] = !PL && xp ? xt[W + lane * VX + v] : R(0);
+        tx[2][v] = !PL && xp ? xt[3 * W + lane * VX + v] : R(0);
+        tx[3][v] = !PL && xp ? xt[4 * W + lane * VX + v] : R(0);
     }
     const bool k1 = w.kappa1 != 0;
     R *rec = nullptr;
@@ -538,7 +549,9 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
     };
     using Yes = std::true_type;
     using No = std::false_type;
-    if (dru) {
+    if constexpr (PL) {
+        run(No{}, No{}, std::bool_constant<D>{});
+    } else if (dru) {
         if (xp && yp) run(Yes{}, Yes{}, Yes{});
         else if (xp) run(Yes{}, No{}, Yes{});
         else if (yp) run(No{}, Yes{}, Yes{});
@@ -559,7 +572,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
         stv(out.Ez + q, ez[r]);
         stv(out.Hx + q, hx[r]);
         stv(out.Hy + q, hy[r]);
-        if (desr >> r & 1u) {
+        if (D || (!V && desr >> r & 1u)) {
             stv(out.J + d[r], jj[r]);
             if (MODE == 1) {
 #pragma unroll
@@ -570,7 +583,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
                 }
             }
         }
-        if (xp) {
+        if (!PL && xp) {
 #pragma unroll
             for (int v = 0; v < VX; ++v) {
                 const int i = i0 + v;
@@ -582,7 +595,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
                 if (sh >= 0) out.phyx[(long long)j * np2 + sh] = phx[r][v];
             }
         }
-        if (yp) {
+        if (!PL && yp) {
             const int te = slab_e(j, ny, np), th = slab_h(j, ny, np);
             if (te >= 0 && j >= 1 && j <= ny - 2) {
 #pragma unroll
@@ -593,6 +606,16 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
             if (th >= 0) stv(out.phxy + (long long)th * P + i0, phy[r]);
         }
     }
+    };
+    const int lo = max(np, 1), xe = xr + W - 1, ye = yr + nw * RPW - 1;
+    const bool inner = xr >= lo && xe <= nx - 2 - lo && yr - 1 >= lo && ye <= ny - 2 - lo &&
+                       !(xr < g.gx0 + g.gnx && xe >= g.gx0 && yr < g.gy0 + g.gny && ye >= g.gy0) &&
+                       !(MODE == 0 && xr < g.sx1 && xe >= g.sx0 && yr < g.sy1 && ye >= g.sy0);
+    const bool invac = xr >= g.dxa + g.dp || xe < g.dxa || yr >= g.dy0 + g.dny || ye < g.dy0;
+    const bool indes = xr >= g.dx0 && xe < g.dx0 + g.dnx && yr >= g.dy0 && ye < g.dy0 + g.dny;
+    if (inner && invac) body(std::true_type{}, std::false_type{});
+    else if (inner && indes) body(std::false_type{}, std::true_type{});
+    else body(std::false_type{}, std::false_type{});
 }
 
 // The Drude coefficients of the pitched design box, in the operations of
@@ -629,14 +652,17 @@ __global__ void k_rt2d_coef(const __grid_constant__ Geo2D g, int slot, const R *
 
 }  // namespace
 
-// A launch's fixed part is about 3 us; a row step is 0.025 us in FP32 (two
-// columns per lane) and 0.24 us in FP64.
+// A wave's fixed part in row steps, fitted to FP32 halos of 4, 6, 8 on seven
+// grids (us per forward step, halo 4 / 6 / 8: 316^2 1.60 / 1.29 / 1.12, 530^2
+// 2.77 / 2.18 / 2.47, 700^2 3.47 / 3.14 / 3.33, 1400^2 8.2 / 7.9 / 9.0, 2048^2
+// 18.0 / 17.4 / 18.3: within 2 % of the best on each), and in FP64 from 3 us of
+// launch against 0.24 us per row step.
 template <typename R>
 Rt2DPlan rt2d_plan(int nx, int ny, int sms, int steps)
 {
     using D = Shape<R>;
     constexpr bool F64 = sizeof(R) == 8;
-    return rt_tile_plan(nx, ny, sms, D::W, D::RPW, D::MAXW, !F64 && steps > 4 ? RT2D_MAX : 4, F64 ? 10.0 : 130.0);
+    return rt_tile_plan(nx, ny, sms, D::W, D::RPW, D::MAXW, !F64 && steps > 4 ? RT2D_MAX : 4, F64 ? 10.0 : 350.0);
 }
 
 template <typename R>

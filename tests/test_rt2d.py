@@ -51,6 +51,8 @@ CASES = [
     ("f32", dict(nx=600, ny=300, npml=10, gap=(17, 17), design=(300, 60), src_offset=80, nsteps=301)),
     ("f32", dict(nx=650, ny=241, pml_kappa_max=2.0, pml_alpha_max=1e3, courant=0.25, eps_s=1.7, eps_g=1.3, nsteps=500, src_offset=90)),
     ("f32", dict(nx=601, ny=270, npml=0, design=(601, 270), src_offset=100, nsteps=301)),
+    # many tiles, most of them of the background or of the design box alone
+    ("f32", dict(nx=1501, ny=1420, npml=10, design=(700, 150), src_offset=610, nsteps=301, snapshot_every=50)),
 ]
 
 
