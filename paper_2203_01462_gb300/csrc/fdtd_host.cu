@@ -421,6 +421,7 @@ Coef<R> make_coef(const fdtd_config &c, double dt, double sigma_max, double gamm
     k.eps_sub = (R)c.sub_eps;
     k.inv_eps_s = (R)(1.0 / c.eps_s);
     k.inv_eps_g = (R)(1.0 / c.eps_g);
+    k.inv_eps_sub = (R)(1.0 / c.sub_eps);
     k.d_eps = (R)(c.eps_inf - c.eps_s);
     k.psi = (R)psi;
     k.psi_s = (R)(c.psi_s_ratio * psi);

@@ -49,7 +49,7 @@ template <typename R>
 struct Coef {
     R S;            // Courant number c0 dt / dx
     R eps_s, eps_g, inv_eps_s, inv_eps_g;
-    R eps_sub;      // 3D: background below the substrate plane
+    R eps_sub, inv_eps_sub;  // 3D: background below the substrate plane
     R d_eps;        // eps_inf - eps_s
     R psi, psi_s;   // scaled psi of the metal and of the background
     R sig_max;      // scaled sigma_max, times 4 for the peak-normalised form

@@ -9,7 +9,8 @@
 // units, see Coef).  Curl component c uses the cyclic axes a = c+1, b = c+2:
 // curl_c = d_a F_b - d_b F_a, each derivative with its own CPML term in the
 // slab of its axis.  Each thread owns four x-adjacent nodes (32 x 8 x 2-node
-// blocks) and runs one vector code path everywhere: next to the PEC walls
+// blocks; FP64: one, 8 x 4-node blocks) and runs one vector code path
+// everywhere: next to the PEC walls
 // it skips the neighbour loads that fall outside the grid and masks the
 // components that are not updated there (H_c exists where p <= n-2 along
 // both of its derivative axes; E_c is updated where p <= n-2 along c and
@@ -23,6 +24,7 @@
 // three components into the node's FP64 accumulator.
 
 #include <algorithm>
+#include <type_traits>
 
 #include "coef_slots.cuh"
 #include "fdtd_internal.h"
@@ -43,8 +45,30 @@ namespace {
 // forward step: 5 blocks everywhere 242.6 us, 6 everywhere 229.3, H and
 // forward E at 7 227.4, everything at 7 227.4 (adjoint 465 against 457 at
 // 6), H at 7 with E at 6 231.7.
+// FP64: one node per thread, blocks of one warp on 8 x 4 nodes.  There the
+// two FP64 units of an SM are the bound (16 cycles per instruction, whatever
+// lanes are active), and they should have even shares of full warps: tiles of
+// four nodes per thread gave the 80 x 34 x 40 grid 300 blocks of unequal cost
+// for 152 SMs (the units 31-39 % busy on average, 56-70 % on the busiest SM)
+// with 30 % of the lanes outside the grid.  us per forward / adjoint step,
+// before and now: 80 x 34 x 40 41.0 / 48.1 -> 15.8 / 17.2, 33 x 21 x 29 30.6 /
+// 38.0 -> 9.1 / 10.7, 128^3 269 / 281 -> 168 / 178, 200 x 160 x 120 480 / 506 ->
+// 282 / 301.
+// Other blocks (80 x 34 x 40, 200 x 160 x 120 forward, before S went into the
+// multiply-adds): 8 x 4 x 1 17.6, 325; 8 x 4 x 2 18.0, 326; 16 x 2 x 1 17.5,
+// 355; 16 x 4 x 2 20.3, 356; 32 x 2 x 1 23.5, 424.  Letting the next launch
+// start early (griddepcontrol.launch_dependents) upset the even placement:
+// 24.8 us.
 constexpr int VX = 4, TBX = 8, TBY = 8, TBZ = 2;
 constexpr int TX = TBX * VX;
+struct Tile4 {
+    static constexpr int N = VX, BX = TBX, BY = TBY, BZ = TBZ;
+};
+struct Tile1 {
+    static constexpr int N = 1, BX = 8, BY = 4, BZ = 1;
+};
+template <typename R>
+using Step = std::conditional_t<sizeof(R) == 4, Tile4, Tile1>;
 static_assert(WAVE3D_TX == TX && WAVE3D_TY == TBY && WAVE3D_TZ == TBZ, "wavefront tiles are the step tiles");
 
 __device__ __forceinline__ bool in_range(int v, int lo, int n) { return (unsigned)(v - lo) < (unsigned)n; }
@@ -74,6 +98,9 @@ __device__ __forceinline__ void st4(double *p, const double (&o)[4])
     reinterpret_cast<double2 *>(p)[0] = make_double2(o[0], o[1]);
     reinterpret_cast<double2 *>(p)[1] = make_double2(o[2], o[3]);
 }
+// One node per thread (FP64).
+__device__ __forceinline__ void ld4(const double *__restrict__ p, double (&o)[1]) { o[0] = *p; }
+__device__ __forceinline__ void st4(double *p, const double (&o)[1]) { *p = o[0]; }
 // Loads for the persistent wavefront kernel, which reads fields other blocks
 // of the same launch wrote: plain (coherent) global loads, never the
 // read-only path that `const __restrict__` pointers allow.
@@ -87,8 +114,8 @@ __device__ __forceinline__ void ld4c(const double *p, double (&o)[4])
     const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
     o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
 }
-template <bool COH, typename R>
-__device__ __forceinline__ void ldv(const R *p, R (&o)[4])
+template <bool COH, typename R, int N>
+__device__ __forceinline__ void ldv(const R *p, R (&o)[N])
 {
     if constexpr (COH) ld4c(p, o);
     else ld4(p, o);
@@ -113,10 +140,18 @@ __device__ __forceinline__ double tf_fma(double a, double b, double x) { return 
 __device__ __forceinline__ float tf_mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double tf_mul(double a, double b) { return __dmul_rn(a, b); }
 
-template <typename R>
-__device__ __forceinline__ void zero4(R (&o)[4])
+// FP64 runs other tiles in the half-step kernels than in the wavefront
+// kernel: there every rounding is fixed.
+__device__ __forceinline__ float mul64(float a, float b) { return a * b; }
+__device__ __forceinline__ double mul64(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sub64(float a, float b) { return a - b; }
+__device__ __forceinline__ double sub64(double a, double b) { return __dsub_rn(a, b); }
+
+template <typename R, int N>
+__device__ __forceinline__ void zero4(R (&o)[N])
 {
-    o[0] = o[1] = o[2] = o[3] = R(0);
+#pragma unroll
+    for (int v = 0; v < N; ++v) o[v] = R(0);
 }
 
 // Slab index of position p along an axis of n nodes (E: node positions,
@@ -150,17 +185,17 @@ __device__ __forceinline__ long long pidx(const Geo3D &g, int ax, int s, int i, 
 // overlap; the pairs of further axes (edges and corners of the shell) are
 // loaded where they are used.  Only one pair is held across the field
 // loads, not all six.
-template <bool HALF>
-__device__ __forceinline__ void slab_x(const Geo3D &g, int i0, int (&sx)[4])
+template <bool HALF, int N>
+__device__ __forceinline__ void slab_x(const Geo3D &g, int i0, int (&sx)[N])
 {
 #pragma unroll
-    for (int v = 0; v < 4; ++v)  // nodes past the last one are row padding: no slab
+    for (int v = 0; v < N; ++v)  // nodes past the last one are row padding: no slab
         sx[v] = i0 + v >= g.n[0] ? -1 : (HALF ? slabH(i0 + v, g.n[0], g.npml) : slabE(i0 + v, g.n[0], g.npml));
 }
 
-template <typename R, bool COH, int AX>
+template <typename R, bool COH, int AX, int N>
 __device__ __forceinline__ void cpml_load_axis(const Geo3D &g, R *const (&psi)[3][2], int i0, int j, int k, int sy,
-                                               int sz, const int (&sx)[4], R (&p)[2][4])
+                                               int sz, const int (&sx)[N], R (&p)[2][N])
 {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -168,7 +203,7 @@ __device__ __forceinline__ void cpml_load_axis(const Geo3D &g, R *const (&psi)[3
         zero4(p[h]);
         if (AX == 0) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v)
+            for (int v = 0; v < N; ++v)
                 if (sx[v] >= 0) p[h][v] = psi[c][h][pidx(g, 0, sx[v], i0 + v, j, k)];
         } else if (AX == 1) {
             if (sy >= 0) ldv<COH>(psi[c][h] + pidx(g, 1, sy, i0, j, k), p[h]);
@@ -179,9 +214,9 @@ __device__ __forceinline__ void cpml_load_axis(const Geo3D &g, R *const (&psi)[3
 }
 
 // The early load: the pair of axis pa (2, 1 or 0).
-template <typename R, bool COH>
+template <typename R, bool COH, int N>
 __device__ __forceinline__ void cpml_preload(const Geo3D &g, R *const (&psi)[3][2], int pa, int i0, int j, int k,
-                                             int sy, int sz, const int (&sx)[4], R (&p)[2][4])
+                                             int sy, int sz, const int (&sx)[N], R (&p)[2][N])
 {
     if (pa == 2) cpml_load_axis<R, COH, 2>(g, psi, i0, j, k, sy, sz, sx, p);
     else if (pa == 1) cpml_load_axis<R, COH, 1>(g, psi, i0, j, k, sy, sz, sx, p);
@@ -190,41 +225,46 @@ __device__ __forceinline__ void cpml_preload(const Geo3D &g, R *const (&psi)[3][
 
 // Axis AX: d[c][h] <- d / kappa (+ the updated psi in the slab of AX) for
 // its two terms, psi stored back.  pre: the pair loaded early when pa == AX.
-template <typename R, bool COH, int AX>
+template <typename R, bool COH, int AX, int N>
 __device__ __forceinline__ void cpml_axis(const Geo3D &g, R *const (&psi)[3][2], const R *const (&tb)[3],
                                           const R *const (&tc)[3], const R *const (&tk)[3], int i0, int j, int k,
-                                          int sy, int sz, const int (&sx)[4], int pa, const R (&pre)[2][4],
-                                          R (&d)[3][2][4])
+                                          int sy, int sz, const int (&sx)[N], int pa, const R (&pre)[2][N],
+                                          R (&d)[3][2][N])
 {
     // with kappa = 1 everywhere the 1/kappa tables are not read (the product
     // by 1 is exact, so the result is the same); coefficient tables are
     // read-only: non-coherent loads, free to move past stores
     const bool k1 = g.kappa1 != 0;
-    R kk[4];
+    R kk[N];
 #pragma unroll
-    for (int v = 0; v < 4; ++v)
+    for (int v = 0; v < N; ++v)
         kk[v] = AX == 0 ? ((!k1 && i0 + v < g.n[0]) ? __ldg(tk[0] + i0 + v) : R(1))
                         : (k1 ? R(1) : __ldg(tk[AX] + (AX == 1 ? j : k)));
-    const bool any = AX == 0 ? (sx[0] >= 0 || sx[1] >= 0 || sx[2] >= 0 || sx[3] >= 0) : (AX == 1 ? sy >= 0 : sz >= 0);
+    bool any = AX == 1 ? sy >= 0 : AX == 2 && sz >= 0;
+    if (AX == 0) {
+#pragma unroll
+        for (int v = 0; v < N; ++v) any |= sx[v] >= 0;
+    }
     if (!any) {
+        if (sizeof(R) == 8 && k1) return;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) d[(AX + 2 - h) % 3][h][v] = d[(AX + 2 - h) % 3][h][v] * kk[v];
+            for (int v = 0; v < N; ++v) d[(AX + 2 - h) % 3][h][v] = mul64(d[(AX + 2 - h) % 3][h][v], kk[v]);
         return;
     }
-    R ps[2][4];
+    R ps[2][N];
     if (pa == AX) {
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) ps[h][v] = pre[h][v];
+            for (int v = 0; v < N; ++v) ps[h][v] = pre[h][v];
     } else {
         cpml_load_axis<R, COH, AX>(g, psi, i0, j, k, sy, sz, sx, ps);
     }
-    R bb[4], cc[4];
+    R bb[N], cc[N];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
+    for (int v = 0; v < N; ++v) {
         if (AX == 0) {
             bb[v] = sx[v] >= 0 ? __ldg(tb[0] + i0 + v) : R(0);
             cc[v] = sx[v] >= 0 ? __ldg(tc[0] + i0 + v) : R(0);
@@ -237,18 +277,29 @@ __device__ __forceinline__ void cpml_axis(const Geo3D &g, R *const (&psi)[3][2],
     for (int h = 0; h < 2; ++h) {
         const int c = (AX + 2 - h) % 3;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
+        for (int v = 0; v < N; ++v) {
             const R dd = d[c][h][v];
-            R t = dd * kk[v];
-            if (AX != 0 || sx[v] >= 0) {
-                ps[h][v] = bb[v] * ps[h][v] + cc[v] * dd;
-                t += ps[h][v];
+            R t;
+            if constexpr (sizeof(R) == 8) {
+                t = dd;
+                if (AX != 0 || sx[v] >= 0) {
+                    ps[h][v] = rn_fma(bb[v], ps[h][v], rn_mul(cc[v], dd));
+                    t = k1 ? dd + ps[h][v] : rn_fma(dd, kk[v], ps[h][v]);
+                } else if (!k1) {
+                    t = rn_mul(dd, kk[v]);
+                }
+            } else {
+                t = dd * kk[v];
+                if (AX != 0 || sx[v] >= 0) {
+                    ps[h][v] = bb[v] * ps[h][v] + cc[v] * dd;
+                    t += ps[h][v];
+                }
             }
             d[c][h][v] = t;
         }
         if (AX == 0) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v)
+            for (int v = 0; v < N; ++v)
                 if (sx[v] >= 0) psi[c][h][pidx(g, 0, sx[v], i0 + v, j, k)] = ps[h][v];
         } else {
             st4(psi[c][h] + pidx(g, AX, AX == 1 ? sy : sz, i0, j, k), ps[h]);
@@ -256,12 +307,30 @@ __device__ __forceinline__ void cpml_axis(const Geo3D &g, R *const (&psi)[3][2],
     }
 }
 
-// All three axes (z, y, x), then out[c] = S (t_a - t_b).
-template <typename R, bool COH>
+// S (a) in FP32.  In FP64 the curl stays unscaled and S goes into the
+// update's multiply-add (hadd, and S / eps in the E half step): three of
+// fifteen operations less per half step where the FP64 units are the bound,
+// the same bits for a Courant number that is a power of two.
+template <typename R>
+__device__ __forceinline__ R scaled(R S, R a)
+{
+    if constexpr (sizeof(R) == 8) return a;
+    else return rn_mul(S, a);
+}
+// h - S curl, of the curl as scaled() left it.
+template <typename R>
+__device__ __forceinline__ R hsub(R S, R cu, R h)
+{
+    if constexpr (sizeof(R) == 8) return rn_fma(-S, cu, h);
+    else return rn_sub(h, cu);
+}
+
+// All three axes (z, y, x), then out[c] = S (t_a - t_b) (FP64: unscaled).
+template <typename R, bool COH, int N>
 __device__ __forceinline__ void cpml_curl(const Geo3D &g, R *const (&psi)[3][2], const R *const (&tb)[3],
                                           const R *const (&tc)[3], const R *const (&tk)[3], int i0, int j, int k,
-                                          int sy, int sz, const int (&sx)[4], int pa, const R (&pre)[2][4], R S,
-                                          R (&d)[3][2][4], R (&out)[3][4])
+                                          int sy, int sz, const int (&sx)[N], int pa, const R (&pre)[2][N], R S,
+                                          R (&d)[3][2][N], R (&out)[3][N])
 {
     cpml_axis<R, COH, 2>(g, psi, tb, tc, tk, i0, j, k, sy, sz, sx, pa, pre, d);
     cpml_axis<R, COH, 1>(g, psi, tb, tc, tk, i0, j, k, sy, sz, sx, pa, pre, d);
@@ -269,7 +338,7 @@ __device__ __forceinline__ void cpml_curl(const Geo3D &g, R *const (&psi)[3][2],
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) out[c][v] = rn_mul(S, d[c][0][v] - d[c][1][v]);
+        for (int v = 0; v < N; ++v) out[c][v] = scaled(S, sub64(d[c][0][v], d[c][1][v]));
 }
 
 // H half step, four x-adjacent nodes per thread:
@@ -279,28 +348,29 @@ __device__ __forceinline__ void cpml_curl(const Geo3D &g, R *const (&psi)[3][2],
 // One tile (bx, by, bz) of the H half step.  COH: loads for the wavefront
 // kernel; FOLD: inc (may then be null) is the plane wave's incident row of
 // this step, whose face corrections are added before the stores.
-template <typename R, bool COH, bool FOLD>
+template <class SH, typename R, bool COH, bool FOLD>
 __device__ __forceinline__ void h_tile(const Geo3D &g, const State3D<R> &s, const Coef<R> &c, const Pml3D<R> &pm,
                                        int bx, int by, int bz, const R *inc)
 {
-    const int i0 = (bx * TBX + threadIdx.x) * VX, j = by * TBY + threadIdx.y, k = bz * TBZ + threadIdx.z;
+    constexpr int N = SH::N;
+    const int i0 = (bx * SH::BX + threadIdx.x) * N, j = by * SH::BY + threadIdx.y, k = bz * SH::BZ + threadIdx.z;
     const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
     if (i0 >= n0 || j >= n1 || k >= n2) return;
     const long long q = k * g.PP + (long long)j * g.px + i0;
     const long long P = g.px, PP = g.PP;
-    const bool yin = j <= n1 - 2, zin = k <= n2 - 2, xin = i0 + VX <= n0 - 1;  // next row / plane / node exist
+    const bool yin = j <= n1 - 2, zin = k <= n2 - 2, xin = i0 + N <= n0 - 1;  // next row / plane / node exist
     const int np = g.npml;
     const int sy = slabH(j, n1, np), sz = slabH(k, n2, np);
-    const bool xslab = i0 < np || i0 + VX - 1 >= n0 - 1 - np;
+    const bool xslab = i0 < np || i0 + N - 1 >= n0 - 1 - np;
     const bool pml = xslab || sy >= 0 || sz >= 0;
-    int sx[4], pa = 0;
-    R pre[2][4];
+    int sx[N], pa = 0;
+    R pre[2][N];
     if (pml) {
         slab_x<true>(g, i0, sx);
         pa = sz >= 0 ? 2 : (sy >= 0 ? 1 : 0);
         cpml_preload<R, COH>(g, s.ph, pa, i0, j, k, sy, sz, sx, pre);
     }
-    R ex[4], exN[4], exU[4], ey[4], eyU[4], ez[4], ezN[4], hx[4], hy[4], hz[4];
+    R ex[N], exN[N], exU[N], ey[N], eyU[N], ez[N], ezN[N], hx[N], hy[N], hz[N];
     ldv<COH>(s.E[0] + q, ex);
     ldv<COH>(s.E[1] + q, ey);
     ldv<COH>(s.E[2] + q, ez);
@@ -321,46 +391,46 @@ __device__ __forceinline__ void h_tile(const Geo3D &g, const State3D<R> &s, cons
     ldv<COH>(s.H[0] + q, hx);
     ldv<COH>(s.H[1] + q, hy);
     ldv<COH>(s.H[2] + q, hz);
-    const R eyE = xin ? s.E[1][q + VX] : R(0), ezE = xin ? s.E[2][q + VX] : R(0);
+    const R eyE = xin ? s.E[1][q + N] : R(0), ezE = xin ? s.E[2][q + N] : R(0);
     const R S = c.S;
-    R cu[3][4];
+    R cu[3][N];
     if (!pml) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const R ezx = v < 3 ? ez[v + 1] : ezE, eyx = v < 3 ? ey[v + 1] : eyE;
-            cu[0][v] = rn_mul(S, (ezN[v] - ez[v]) - (eyU[v] - ey[v]));
-            cu[1][v] = rn_mul(S, (exU[v] - ex[v]) - (ezx - ez[v]));
-            cu[2][v] = rn_mul(S, (eyx - ey[v]) - (exN[v] - ex[v]));
+        for (int v = 0; v < N; ++v) {
+            const R ezx = v < N - 1 ? ez[v < N - 1 ? v + 1 : v] : ezE, eyx = v < N - 1 ? ey[v < N - 1 ? v + 1 : v] : eyE;
+            cu[0][v] = scaled(S, (ezN[v] - ez[v]) - (eyU[v] - ey[v]));
+            cu[1][v] = scaled(S, (exU[v] - ex[v]) - (ezx - ez[v]));
+            cu[2][v] = scaled(S, (eyx - ey[v]) - (exN[v] - ex[v]));
         }
     } else {
-        R d[3][2][4];  // d[c][0]: along c+1, d[c][1]: along c+2 (forward differences of E)
+        R d[3][2][N];  // d[c][0]: along c+1, d[c][1]: along c+2 (forward differences of E)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
+        for (int v = 0; v < N; ++v) {
             d[0][0][v] = ezN[v] - ez[v];                         // d_y Ez
             d[0][1][v] = eyU[v] - ey[v];                         // d_z Ey
             d[1][0][v] = exU[v] - ex[v];                         // d_z Ex
-            d[1][1][v] = (v < 3 ? ez[v + 1] : ezE) - ez[v];      // d_x Ez
-            d[2][0][v] = (v < 3 ? ey[v + 1] : eyE) - ey[v];      // d_x Ey
+            d[1][1][v] = (v < N - 1 ? ez[v < N - 1 ? v + 1 : v] : ezE) - ez[v];      // d_x Ez
+            d[2][0][v] = (v < N - 1 ? ey[v < N - 1 ? v + 1 : v] : eyE) - ey[v];      // d_x Ey
             d[2][1][v] = exN[v] - ex[v];                         // d_y Ex
         }
         cpml_curl<R, COH>(g, s.ph, pm.bH, pm.cH, pm.kiH, i0, j, k, sy, sz, sx, pa, pre, S, d, cu);
     }
     if (xin && yin && zin) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            hx[v] = rn_sub(hx[v], cu[0][v]);
-            hy[v] = rn_sub(hy[v], cu[1][v]);
-            hz[v] = rn_sub(hz[v], cu[2][v]);
+        for (int v = 0; v < N; ++v) {
+            hx[v] = hsub(S, cu[0][v], hx[v]);
+            hy[v] = hsub(S, cu[1][v], hy[v]);
+            hz[v] = hsub(S, cu[2][v], hz[v]);
         }
     } else {
         // last row / plane / node: H_x exists where j, k <= n-2, H_y where
         // k, i <= n-2, H_z where i, j <= n-2 (nodes past n0 are padding)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
+        for (int v = 0; v < N; ++v) {
             const int i = i0 + v;
-            if (yin && zin && i < n0) hx[v] = rn_sub(hx[v], cu[0][v]);
-            if (zin && i <= n0 - 2) hy[v] = rn_sub(hy[v], cu[1][v]);
-            if (yin && i <= n0 - 2) hz[v] = rn_sub(hz[v], cu[2][v]);
+            if (yin && zin && i < n0) hx[v] = hsub(S, cu[0][v], hx[v]);
+            if (zin && i <= n0 - 2) hy[v] = hsub(S, cu[1][v], hy[v]);
+            if (yin && i <= n0 - 2) hz[v] = hsub(S, cu[2][v], hz[v]);
         }
     }
     if constexpr (FOLD) {
@@ -371,13 +441,13 @@ __device__ __forceinline__ void h_tile(const Geo3D &g, const State3D<R> &s, cons
             if ((k == lz - 1 || k == uz) && j >= ly && j <= uy) {
                 const R a = k == uz ? -S : S, e = k == uz ? inc[uz - lz] : inc[0];
 #pragma unroll
-                for (int v = 0; v < 4; ++v)
+                for (int v = 0; v < N; ++v)
                     if (i0 + v >= lx && i0 + v < ux) hy[v] = tf_fma(a, e, hy[v]);
             }
             if ((j == ly - 1 || j == uy) && k >= lz && k <= uz) {
                 const R a = j == uy ? S : -S, e = inc[k - lz];
 #pragma unroll
-                for (int v = 0; v < 4; ++v)
+                for (int v = 0; v < N; ++v)
                     if (i0 + v >= lx && i0 + v < ux) hz[v] = tf_fma(a, e, hz[v]);
             }
         }
@@ -390,12 +460,12 @@ __device__ __forceinline__ void h_tile(const Geo3D &g, const State3D<R> &s, cons
 // The H half step of the whole grid, bottom up or (zrev) top down; FOLD:
 // with the plane wave's H-face corrections of incident row inc.
 template <typename R, bool FOLD>
-__global__ void __launch_bounds__(TBX *TBY *TBZ, sizeof(R) == 4 ? 6 : 1)
+__global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(R) == 4 ? 6 : 24)
     k_h3d(Geo3D g, State3D<R> s, int slot, Pml3D<R> pm, int zrev, const R *inc)
 {
     wait_previous_grid();
     const int bz = zrev ? gridDim.z - 1 - blockIdx.z : blockIdx.z;
-    h_tile<R, false, FOLD>(g, s, coef_at<R>(slot), pm, blockIdx.x, blockIdx.y, bz, inc);
+    h_tile<Step<R>, R, false, FOLD>(g, s, coef_at<R>(slot), pm, blockIdx.x, blockIdx.y, bz, inc);
 }
 
 // E half step: curl H with backward differences (CPML terms as in the H
@@ -404,28 +474,29 @@ __global__ void __launch_bounds__(TBX *TBY *TBZ, sizeof(R) == 4 ? 6 : 1)
 // One tile (bx, by, bz) of the E half step.  COH: loads for the wavefront
 // kernel; FOLD (forward): the plane wave's face corrections of row
 // a3.tf_inc (when set) added before the stores.
-template <typename R, int MODE, bool COH, bool FOLD>
+template <class SH, typename R, int MODE, bool COH, bool FOLD>
 __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, const Coef<R> &c, const Pml3D<R> &pm,
                                        const Step3D<R> &a3, int bx, int by, int bz)
 {
-    const int x0 = bx * TX, y0 = by * TBY, z0 = bz * TBZ;
-    const int i0 = x0 + threadIdx.x * VX, j = y0 + threadIdx.y, k = z0 + threadIdx.z;
+    constexpr int N = SH::N, TX = SH::BX * N, TY = SH::BY, TZ = SH::BZ;
+    const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ;
+    const int i0 = x0 + threadIdx.x * N, j = y0 + threadIdx.y, k = z0 + threadIdx.z;
     const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
     if (i0 >= n0 || j >= n1 || k >= n2) return;
     const long long q = k * g.PP + (long long)j * g.px + i0;
     const long long P = g.px, PP = g.PP;
     const int np = g.npml;
     const int sy = slabE(j, n1, np), sz = slabE(k, n2, np);
-    const bool xslab = i0 < np || i0 + VX - 1 >= n0 - np;
+    const bool xslab = i0 < np || i0 + N - 1 >= n0 - np;
     const bool pml = xslab || sy >= 0 || sz >= 0;
-    int sx[4], pa = 0;
-    R pre[2][4];
+    int sx[N], pa = 0;
+    R pre[2][N];
     if (pml) {
         slab_x<false>(g, i0, sx);
         pa = sz >= 0 ? 2 : (sy >= 0 ? 1 : 0);
         cpml_preload<R, COH>(g, s.pe, pa, i0, j, k, sy, sz, sx, pre);
     }
-    R hx[4], hxS[4], hxD[4], hy[4], hyD[4], hz[4], hzS[4], e[3][4];
+    R hx[N], hxS[N], hxD[N], hy[N], hyD[N], hz[N], hzS[N], e[3][N];
     ldv<COH>(s.H[0] + q, hx);
     ldv<COH>(s.H[1] + q, hy);
     ldv<COH>(s.H[2] + q, hz);
@@ -449,31 +520,31 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
     ldv<COH>(s.E[0] + q, e[0]);
     ldv<COH>(s.E[1] + q, e[1]);
     ldv<COH>(s.E[2] + q, e[2]);
-    R curl[3][4];
+    R curl[3][N];
     if (!pml) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const R hyx = v > 0 ? hy[v - 1] : hyW, hzx = v > 0 ? hz[v - 1] : hzW;
-            curl[0][v] = rn_mul(c.S, (hz[v] - hzS[v]) - (hy[v] - hyD[v]));
-            curl[1][v] = rn_mul(c.S, (hx[v] - hxD[v]) - (hz[v] - hzx));
-            curl[2][v] = rn_mul(c.S, (hy[v] - hyx) - (hx[v] - hxS[v]));
+        for (int v = 0; v < N; ++v) {
+            const R hyx = v > 0 ? hy[v > 0 ? v - 1 : 0] : hyW, hzx = v > 0 ? hz[v > 0 ? v - 1 : 0] : hzW;
+            curl[0][v] = scaled(c.S, (hz[v] - hzS[v]) - (hy[v] - hyD[v]));
+            curl[1][v] = scaled(c.S, (hx[v] - hxD[v]) - (hz[v] - hzx));
+            curl[2][v] = scaled(c.S, (hy[v] - hyx) - (hx[v] - hxS[v]));
         }
     } else {
-        R d[3][2][4];  // backward differences of H
+        R d[3][2][N];  // backward differences of H
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
+        for (int v = 0; v < N; ++v) {
             d[0][0][v] = hz[v] - hzS[v];                         // d_y Hz
             d[0][1][v] = hy[v] - hyD[v];                         // d_z Hy
             d[1][0][v] = hx[v] - hxD[v];                         // d_z Hx
-            d[1][1][v] = hz[v] - (v > 0 ? hz[v - 1] : hzW);      // d_x Hz
-            d[2][0][v] = hy[v] - (v > 0 ? hy[v - 1] : hyW);      // d_x Hy
+            d[1][1][v] = hz[v] - (v > 0 ? hz[v > 0 ? v - 1 : 0] : hzW);      // d_x Hz
+            d[2][0][v] = hy[v] - (v > 0 ? hy[v > 0 ? v - 1 : 0] : hyW);      // d_x Hy
             d[2][1][v] = hx[v] - hxS[v];                         // d_y Hx
         }
         cpml_curl<R, COH>(g, s.pe, pm.bE, pm.cE, pm.kiE, i0, j, k, sy, sz, sx, pa, pre, c.S, d, curl);
     }
     // E_c is updated where p <= n-2 along c and 1 <= p <= n-2 across; a
     // component that is not updated keeps its value (zero on the walls).
-    const bool full = i0 >= 1 && i0 + VX <= n0 - 1 && j >= 1 && j <= n1 - 2 && k >= 1 && k <= n2 - 2;
+    const bool full = i0 >= 1 && i0 + N <= n0 - 1 && j >= 1 && j <= n1 - 2 && k >= 1 && k <= n2 - 2;
     const bool jmid = j >= 1 && j <= n1 - 2, kmid = k >= 1 && k <= n2 - 2;
     auto upd = [&](int cc, int v) -> bool {
         const int i = i0 + v;
@@ -483,13 +554,17 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
         return k <= n2 - 2 && imid && jmid;
     };
     const bool touches = (x0 < g.d0[0] + g.dn[0] && x0 + TX > g.d0[0] && y0 < g.d0[1] + g.dn[1] &&
-                          y0 + TBY > g.d0[1] && z0 < g.d0[2] + g.dn[2] && z0 + TBZ > g.d0[2]) ||
-                         (MODE == 0 && x0 < g.s1[0] && x0 + TX > g.s0[0] && y0 < g.s1[1] && y0 + TBY > g.s0[1] &&
-                          z0 < g.s1[2] && z0 + TBZ > g.s0[2]);
-    const R inv_bg = rcp(k < g.sub_hi ? c.eps_sub : c.eps_s);
+                          y0 + TY > g.d0[1] && z0 < g.d0[2] + g.dn[2] && z0 + TZ > g.d0[2]) ||
+                         (MODE == 0 && x0 < g.s1[0] && x0 + TX > g.s0[0] && y0 < g.s1[1] && y0 + TY > g.s0[1] &&
+                          z0 < g.s1[2] && z0 + TZ > g.s0[2]);
+    // (FP64 reciprocals, some fifteen operations, come from the host; FP32's
+    // are rounded from FP32 operands)
+    constexpr bool F64 = sizeof(R) == 8;
+    const R inv_bg = F64 ? (k < g.sub_hi ? c.inv_eps_sub : c.inv_eps_s) : rcp(k < g.sub_hi ? c.eps_sub : c.eps_s);
+    const R f_bg = F64 ? c.S * inv_bg : inv_bg;  // the background's factor of the curl
     // the E-face corrections of the plane wave (see the TFSF notes; the
     // faces lie in background material)
-    auto tf_fix = [&](int cc, R(&x)[4]) {
+    auto tf_fix = [&](int cc, R(&x)[N]) {
         if constexpr (FOLD && MODE == 0) {
             if (!a3.tf_inc) return;
             const int lx = g.tf_lo[0], ly = g.tf_lo[1], lz = g.tf_lo[2];
@@ -498,12 +573,12 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
             if (cc == 0 && (k == lz || k == uz) && j >= ly && j <= uy) {
                 const R m = tf_mul(k == uz ? -c.S : c.S, k == uz ? hi[uz - lz + 1] : hi[0]);
 #pragma unroll
-                for (int v = 0; v < 4; ++v)
+                for (int v = 0; v < N; ++v)
                     if (i0 + v >= lx && i0 + v < ux) x[v] = tf_fma(m, inv_bg, x[v]);
             }
             if (cc == 2 && j >= ly && j <= uy && k >= lz && k < uz) {
 #pragma unroll
-                for (int v = 0; v < 4; ++v)
+                for (int v = 0; v < N; ++v)
                     if (i0 + v == lx || i0 + v == ux)
                         x[v] = tf_fma(tf_mul(i0 + v == ux ? c.S : -c.S, hi[k - lz + 1]), inv_bg, x[v]);
             }
@@ -513,8 +588,8 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
 #pragma unroll
         for (int cc = 0; cc < 3; ++cc) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v)
-                if (full || upd(cc, v)) e[cc][v] = rn_fma(curl[cc][v], inv_bg, e[cc][v]);
+            for (int v = 0; v < N; ++v)
+                if (full || upd(cc, v)) e[cc][v] = rn_fma(curl[cc][v], f_bg, e[cc][v]);
             tf_fix(cc, e[cc]);
             st4(s.E[cc] + q, e[cc]);
         }
@@ -527,12 +602,12 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
     const long long d0 = ((long long)(k - g.d0[2]) * g.dn[1] + (j - g.d0[1])) * g.dp + (i0 - g.dxa);
     const bool rgap = in_range(j, g.g0[1], g.gn[1]) && in_range(k, g.g0[2], g.gn[2]);
     const bool rsrc = MODE == 0 && in_range(j, g.s0[1], g.s1[1] - g.s0[1]) && in_range(k, g.s0[2], g.s1[2] - g.s0[2]);
-    R rt4[4] = {R(0), R(0), R(0), R(0)}, J4[3][4], em4[3][4];
-    double G4[4] = {0.0, 0.0, 0.0, 0.0}, gadd[4] = {0.0, 0.0, 0.0, 0.0};
+    R rt4[N] = {}, J4[3][N], em4[3][N];
+    double G4[N] = {}, gadd[N] = {};
 #pragma unroll
     for (int cc = 0; cc < 3; ++cc)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) J4[cc][v] = em4[cc][v] = R(0);
+        for (int v = 0; v < N; ++v) J4[cc][v] = em4[cc][v] = R(0);
     if (vdes) {
         ld4(a3.rho_t + d0, rt4);
 #pragma unroll
@@ -545,9 +620,9 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
     const R src_fwd = (MODE == 0 && rsrc) ? *a3.src : R(0);
 #pragma unroll
     for (int cc = 0; cc < 3; ++cc) {
-        R en[4], jn4[4];
+        R en[N], jn4[N];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
+        for (int v = 0; v < N; ++v) {
             const int i = i0 + v;
             const bool gap = rgap && in_range(i, g.g0[0], g.gn[0]);
             const int gidx = ((k - g.g0[2]) * g.gn[1] + (j - g.g0[1])) * g.gn[0] + (i - g.g0[0]);
@@ -562,24 +637,48 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
                 en[v] = e[cc][v];
             } else if (vdes && in_range(i, g.d0[0], g.dn[0]) && !gap) {
                 const R rt = rt4[v];
-                const R eps = c.eps_s + rt * c.d_eps;
-                const R psi = c.psi_s + rt * (c.psi - c.psi_s);
-                const R sig = c.sig_max * rt * (R(1) - rt);
+                R eps = c.eps_s + rt * c.d_eps;
+                R psi = c.psi_s + rt * (c.psi - c.psi_s);
+                R sig = c.sig_max * rt * (R(1) - rt);
+                if constexpr (F64) {
+                    eps = rn_fma(rt, c.d_eps, c.eps_s);
+                    psi = rn_fma(rt, c.psi - c.psi_s, c.psi_s);
+                    sig = rn_mul(rn_mul(c.sig_max, rt), R(1) - rt);
+                }
                 const R bJ = R(0.5) * psi * c.inv1g;
                 const R hs = R(0.5) * (sig + bJ);
                 const R cb = rcp(eps + hs);
                 const R ca = (eps - hs) * cb;
-                en[v] = ca * e[cc][v] + cb * (curl[cc][v] - c.half1pkJ * J4[cc][v] - src);
-                jn4[v] = c.kJ * J4[cc][v] + bJ * (en[v] + e[cc][v]);
+                if constexpr (F64) {
+                    const R x = rn_fma(-c.half1pkJ, J4[cc][v], rn_mul(c.S, curl[cc][v])) - src;
+                    en[v] = rn_fma(cb, x, rn_mul(ca, e[cc][v]));
+                    jn4[v] = rn_fma(c.kJ, J4[cc][v], rn_mul(bJ, en[v] + e[cc][v]));
+                } else {
+                    en[v] = ca * e[cc][v] + cb * (curl[cc][v] - c.half1pkJ * J4[cc][v] - src);
+                    jn4[v] = c.kJ * J4[cc][v] + bJ * (en[v] + e[cc][v]);
+                }
                 if (MODE == 1) {
                     // Eq. (25a-c) folded through the chain rule of Eq. (27).
-                    const R term = -c.t_eps * (en[v] - e[cc][v]) -
-                                   c.t_sig * (R(1) - R(2) * rt) * R(0.5) * (en[v] + e[cc][v]) -
-                                   c.t_dpsi * rcp(psi) * R(0.5) * (jn4[v] + J4[cc][v]);
-                    gadd[v] += (double)em4[cc][v] * (double)term;
+                    if constexpr (F64) {
+                        const R a1 = rn_mul(c.t_sig, rn_fma(R(-2), rt, R(1))) * R(0.5), a2 = rn_mul(c.t_dpsi, rcp(psi)) * R(0.5);
+                        R term = rn_mul(-c.t_eps, en[v] - e[cc][v]);
+                        term = rn_fma(-a1, en[v] + e[cc][v], term);
+                        term = rn_fma(-a2, jn4[v] + J4[cc][v], term);
+                        gadd[v] = rn_fma(em4[cc][v], term, gadd[v]);
+                    } else {
+                        const R term = -c.t_eps * (en[v] - e[cc][v]) -
+                                       c.t_sig * (R(1) - R(2) * rt) * R(0.5) * (en[v] + e[cc][v]) -
+                                       c.t_dpsi * rcp(psi) * R(0.5) * (jn4[v] + J4[cc][v]);
+                        gadd[v] += (double)em4[cc][v] * (double)term;
+                    }
                 }
             } else {
-                en[v] = rn_fma(curl[cc][v] - src, gap ? rcp(c.eps_g) : inv_bg, e[cc][v]);
+                if constexpr (F64) {  // (as in a tile without design box where there is no source)
+                    if (src == R(0)) en[v] = rn_fma(curl[cc][v], gap ? rn_mul(c.S, c.inv_eps_g) : f_bg, e[cc][v]);
+                    else en[v] = rn_fma(rn_sub(rn_mul(c.S, curl[cc][v]), src), gap ? c.inv_eps_g : inv_bg, e[cc][v]);
+                } else {
+                    en[v] = rn_fma(curl[cc][v] - src, gap ? rcp(c.eps_g) : inv_bg, e[cc][v]);
+                }
             }
             if (MODE == 0 && gap && a3.gap_rec && (full || upd(cc, v)))
                 a3.gap_rec[(long long)cc * g.Mg + gidx] = en[v];
@@ -593,18 +692,18 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
     }
     if (MODE == 1 && vdes) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) G4[v] += gadd[v];
+        for (int v = 0; v < N; ++v) G4[v] += gadd[v];
         st4(a3.G + d0, G4);
     }
 }
 
 template <typename R, int MODE, bool FOLD>
-__global__ void __launch_bounds__(TBX *TBY *TBZ, sizeof(R) == 4 ? (MODE == 1 ? 6 : 7) : 1)
+__global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(R) == 4 ? (MODE == 1 ? 6 : 7) : 24)
     k_e3d(Geo3D g, State3D<R> s, int slot, Pml3D<R> pm, Step3D<R> a3, int zrev)
 {
     wait_previous_grid();
     const int bz = zrev ? gridDim.z - 1 - blockIdx.z : blockIdx.z;
-    e_tile<R, MODE, false, FOLD>(g, s, coef_at<R>(slot), pm, a3, blockIdx.x, blockIdx.y, bz);
+    e_tile<Step<R>, R, MODE, false, FOLD>(g, s, coef_at<R>(slot), pm, a3, blockIdx.x, blockIdx.y, bz);
 }
 
 // ------------------------------------------------ plane wave (TFSF notes)
@@ -759,7 +858,7 @@ __global__ void __launch_bounds__(TBX *TBY *TBZ, sizeof(R) == 4 ? WAVE_MINB : 1)
         if (!isE) {
             const R *inc = (MODE == 0 && w.tf) ? w.tf + (long long)(w.n0 + t) * w.tf_row : nullptr;
 #pragma unroll 1
-            for (int bx = bx0; bx < bx1; ++bx) h_tile<R, true, true>(g, s, c, pm, bx, by, sl, inc);
+            for (int bx = bx0; bx < bx1; ++bx) h_tile<Tile4, R, true, true>(g, s, c, pm, bx, by, sl, inc);
         } else {
             Step3D<R> a = a0;
             if (MODE == 0) {
@@ -774,7 +873,7 @@ __global__ void __launch_bounds__(TBX *TBY *TBZ, sizeof(R) == 4 ? WAVE_MINB : 1)
                 a.rec = w.rec + (long long)(m - 1 - w.rec0) * 3 * g.Mdi;
             }
 #pragma unroll 1
-            for (int bx = bx0; bx < bx1; ++bx) e_tile<R, MODE, true, true>(g, s, c, pm, a, bx, by, sl);
+            for (int bx = bx0; bx < bx1; ++bx) e_tile<Tile4, R, MODE, true, true>(g, s, c, pm, a, bx, by, sl);
         }
         __syncthreads();
         // E items of the last step have no reader in this launch
@@ -816,7 +915,10 @@ template <typename R>
 int launch_step3d(int mode, const Geo3D &g, const State3D<R> &s, int c, const Pml3D<R> &pm,
                   const Step3D<R> &a, cudaStream_t st)
 {
-    dim3 vblock(TBX, TBY, TBZ), vgrid((g.n[0] + TX - 1) / TX, (g.n[1] + TBY - 1) / TBY, (g.n[2] + TBZ - 1) / TBZ);
+    using D = Step<R>;
+    constexpr int TX = D::BX * D::N;
+    dim3 vblock(D::BX, D::BY, D::BZ),
+        vgrid((g.n[0] + TX - 1) / TX, (g.n[1] + D::BY - 1) / D::BY, (g.n[2] + D::BZ - 1) / D::BZ);
     // The H half step sweeps the planes upwards and the E half step
     // downwards (blocks start in blockIdx order), so each launch begins where
     // the previous one ended, on planes whose fields are still in L2.  Each
