@@ -6,8 +6,7 @@
 // As im2col + GEMM + col2im + bias passes a training step of the base-24
 // network on 8 x 256^2 maps moved about 25 GB: each im2col matrix is nine
 // times its activations and goes through HBM twice.  Without them the step
-// went from 15.8 to 4.2 ms and a prediction of one map from 0.94 to 0.35 ms
-// (1.04 -> 1.00 ms for a step on one 8 x 8 map, which is launch-bound).  What
+// went from 15.8 to 4.2 ms and a prediction of one map from 0.94 to 0.35 ms.  What
 // bounds these kernels now is instruction issue and shared memory: rounding
 // and staging the operands (the 72 -> 24 convolution at 256^2: 140 us
 // forward, 168 us input gradient, 293 us weight gradient, with 30 to 60 us of
@@ -30,11 +29,20 @@
 // to 80 bytes: ldmatrix and the 16-byte stores hit distinct banks), the next
 // slice's global loads in flight in registers while the current one is
 // multiplied, one barrier per slice.
+//
+// Every kernel here and in nn.cu is launched before its predecessor has ended
+// and waits for it before it touches memory (programmatic dependent launch):
+// a step is about 115 launches, many of a few microseconds.  128^2 x 2 training
+// step 0.98 -> 0.80 ms, 256^2 prediction 0.34 -> 0.25.  The short kernels and
+// the weight gradient, which leaves room on the SMs, also let their
+// successor's blocks in while they run; for the forward and input-gradient
+// kernels that cost the 8 x 256^2 step 1 % (3.55 -> 3.60 ms).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "../../include/surrogate.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -129,6 +137,7 @@ __global__ void __launch_bounds__(32 * WM * WN) k_conv3(const float *__restrict_
                                                         const float *__restrict__ bias, float *out, int ci, int co,
                                                         long long P, int H, int W, int relu, int kc, float *part)
 {
+    fdtd::pdl_wait();
     constexpr int BM = 16 * MF * WM, BN = 32 * WN, NT = 32 * WM * WN, KP = BK / WM, AP = BM * 16 / NT;
     static_assert(BM * 16 % NT == 0, "whole pairs per thread");
     __shared__ __align__(16) __nv_bfloat16 As[2][BM * BKP];
@@ -236,38 +245,71 @@ __global__ void __launch_bounds__(32 * WM * WN) k_conv3(const float *__restrict_
         }
 }
 
-// part[0][e] + part[1][e] + ... + part[S - 1][e] (slices n apart), in that
-// order, sixteen loads in flight.
-__device__ __forceinline__ float slices(const float *__restrict__ part, long long n, long long e, int S)
+// V values from e on of part[0] + part[1] + ... + part[S - 1] (slices n
+// apart), in that order, the loads of eight slices in flight.
+template <int V>
+__device__ __forceinline__ void slices(const float *__restrict__ part, long long n, long long e, int S, float (&a)[V])
 {
-    float a = part[e];
-    for (int z = 1; z < S; z += 16) {
-        float v[16];
+    auto load = [&](long long z, float (&o)[V]) {
+        if constexpr (V == 4) {
+            const float4 t = *reinterpret_cast<const float4 *>(part + z * n + e);
+            o[0] = t.x;
+            o[1] = t.y;
+            o[2] = t.z;
+            o[3] = t.w;
+        } else {
+            o[0] = part[z * n + e];
+        }
+    };
+    constexpr int D = V == 4 ? 8 : 16;
+    load(0, a);
+    for (int z = 1; z < S; z += D) {
+        float v[D][V];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) v[q] = z + q < S ? part[(z + q) * n + e] : 0.0f;
+        for (int q = 0; q < D; ++q)
+            if (z + q < S) load(z + q, v[q]);
 #pragma unroll
-        for (int q = 0; q < 16; ++q)
-            if (z + q < S) a += v[q];
+        for (int q = 0; q < D; ++q)
+            if (z + q < S)
+#pragma unroll
+                for (int i = 0; i < V; ++i) a[i] += v[q][i];
     }
-    return a;
 }
 
-// y = act(sum of the S slices of part, in order, + bias).
-__global__ void k_slices_bias_act(float *y, const float *__restrict__ part, const float *__restrict__ bias, int M,
-                                  long long P, int S, int relu)
+// y = act(sum of the S slices of part, in order, + bias); V divides P.
+template <int V>
+__global__ void __launch_bounds__(128) k_slices_bias_act(float *y, const float *__restrict__ part,
+                                                         const float *__restrict__ bias, int M, long long P, int S,
+                                                         int relu)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     const long long n = (long long)M * P;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const float v = slices(part, n, e, S) + bias[e / P];
-        y[e] = relu && v < 0.0f ? 0.0f : v;
+    for (long long e = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * V; e < n;
+         e += (long long)gridDim.x * blockDim.x * V) {
+        float a[V];
+        slices<V>(part, n, e, S, a);
+        const float b = bias[e / P];
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            a[i] += b;
+            if (relu && a[i] < 0.0f) a[i] = 0.0f;
+        }
+        if constexpr (V == 4) *reinterpret_cast<float4 *>(y + e) = make_float4(a[0], a[1], a[2], a[3]);
+        else y[e] = a[0];
     }
 }
 
 // C = the sum of the S slices of part, in order.
-__global__ void k_slices(float *C, const float *__restrict__ part, long long n, int S)
+__global__ void __launch_bounds__(64) k_slices(float *C, const float *__restrict__ part, long long n, int S)
 {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-        C[e] = slices(part, n, e, S);
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+        float a[1];
+        slices<1>(part, n, e, S, a);
+        C[e] = a[0];
+    }
 }
 
 // Weight gradient: rows = output channels, columns = (c, t), k = pixels.  A
@@ -278,6 +320,8 @@ __global__ void __launch_bounds__(32 * WM * WN) k_conv3_wgrad(const float *__res
                                                               float *gw, int ci, int co, long long P, int H, int W,
                                                               long long kc, float *part)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     constexpr int BM = 16 * MF * WM, BN = 32 * WN, NT = 32 * WM * WN, HW = NT / 16, NB = (BN + HW - 1) / HW,
                   NA = (BM + HW - 1) / HW;
     __shared__ __align__(16) __nv_bfloat16 As[2][BM * BKP];
@@ -406,6 +450,7 @@ __global__ void __launch_bounds__(256, 2)
 k_conv3_fwd_t(const float *__restrict__ x, const float *__restrict__ w, const float *__restrict__ bias, float *y, int ci,
               int co, int B, int H, int W, int relu, int kc, float *part)
 {
+    fdtd::pdl_wait();
     constexpr int ROWS = TH / WM, BM = 16 * MF * WM, CH = 16, KC = 144, AS = KC + 8,
                   XC = ((ROWS + 2) * 3 * RS / 2 + 11) / 32 * 64 + 40,  // channel stride: 20 words mod 32
         XN = (ROWS + 2) / 2, AU = BM * KC / 4, AN = (AU + 255) / 256, AB = MF == 3 ? 2 : 5;
@@ -558,6 +603,7 @@ __global__ void __launch_bounds__(256, 2)
 k_conv3_dgrad_t(const float *__restrict__ dy, const float *__restrict__ w, float *dx, int ci, int co, int Kp, int B, int H,
                 int W, int add)
 {
+    fdtd::pdl_wait();
     constexpr int BM = 16 * MF;
     extern __shared__ __align__(16) unsigned dsm[];
     unsigned *X = dsm;  // [Kp / 2][XCD]
@@ -714,6 +760,8 @@ __global__ void __launch_bounds__(128 * WM) k_conv3_wgrad_t(const float *__restr
                                                             float *gw, int ci, int co, int B, int H, int W, long long kc,
                                                             float *part)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     constexpr int WN = 4, BM = 16 * MF * WM, BN = 128, NT = 128 * WM, CH = 16, XC = 9 * RS,
                   XN = (3 + WM - 1) / WM, AN = BM * 8 / NT;
     static_assert(BM * 8 % NT == 0, "whole units per thread");
@@ -835,9 +883,9 @@ __global__ void __launch_bounds__(128 * WM) k_conv3_wgrad_t(const float *__restr
 
 int status() { return cudaGetLastError() == cudaSuccess ? 0 : 3; }
 
-inline int slice_blocks(long long n)
+inline int slice_blocks(long long n, int per)
 {
-    const long long b = (n + 63) / 64;
+    const long long b = (n + per - 1) / per;
     return (int)(b < 152 * 64 ? b : 152 * 64);
 }
 
@@ -865,7 +913,7 @@ bool fwd_tiled(const float *x, const float *w, const float *bias, float *y, int 
     constexpr size_t smem = (2 * 16 * XC + 2 * BM * 152) * sizeof(__nv_bfloat16);
     if (!smem_ready((const void *)k_conv3_fwd_t<MF, WM>, smem)) return false;
     const dim3 grid((unsigned)((W + 31) / 32 * ((H + ROWS - 1) / ROWS) * B), (co + BM - 1) / BM, splits);
-    k_conv3_fwd_t<MF, WM><<<grid, 256, smem, st>>>(x, w, bias, y, ci, co, B, H, W, relu, kc, part);
+    fdtd::launch_pdl_smem(k_conv3_fwd_t<MF, WM>, grid, 256, smem, st, x, w, bias, y, ci, co, B, H, W, relu, kc, part);
     return true;
 }
 
@@ -875,7 +923,7 @@ void launch(const float *in, const float *w, const float *bias, float *out, int 
 {
     const int M = DG ? ci : co, BM = 16 * MF * WM, BN = 32 * WN;
     const dim3 grid((unsigned)((P + BN - 1) / BN), (M + BM - 1) / BM, splits);
-    k_conv3<MF, WM, WN, DG><<<grid, 32 * WM * WN, 0, st>>>(in, w, bias, out, ci, co, P, H, W, relu, kc, part);
+    fdtd::launch_pdl_smem(k_conv3<MF, WM, WN, DG>, grid, 32 * WM * WN, 0, st, in, w, bias, out, ci, co, P, H, W, relu, kc, part);
 }
 
 // Rows: up to 32 in one 32-row tile, up to 48 in one of 48, else tiles of 96.
@@ -918,7 +966,12 @@ int nn_conv3_fwd(const float *x, const float *w, const float *bias, float *y, in
     if (!(tiled(W) && aligned16(x) && aligned16(y) && aligned16(work) &&
           tile(x, w, bias, y, ci, co, B, H, W, relu, (int)kc, splits, work, st)))
         conv3<false>(x, w, bias, y, ci, co, P, H, W, relu, (int)kc, splits, work, st);
-    if (splits > 1) k_slices_bias_act<<<slice_blocks(co * P), 64, 0, st>>>(y, work, bias, co, P, splits, relu);
+    if (splits > 1) {
+        if (P % 4 == 0 && aligned16(y) && aligned16(work))
+            fdtd::launch_pdl_smem(k_slices_bias_act<4>, slice_blocks(co * P, 512), 128, 0, st, y, work, bias, co, P, splits, relu);
+        else
+            fdtd::launch_pdl_smem(k_slices_bias_act<1>, slice_blocks(co * P, 128), 128, 0, st, y, work, bias, co, P, splits, relu);
+    }
     return status();
 }
 
@@ -934,7 +987,7 @@ int nn_conv3_dgrad(const float *dy, const float *w, float *dx, int ci, int co, i
                             : (G == 9 ? k_conv3_dgrad_t<3, 9> : G == 3 ? k_conv3_dgrad_t<3, 3> : k_conv3_dgrad_t<3, 1>);
     if (tiled(W) && aligned16(dy) && aligned16(dx) && smem_ready((const void *)f, smem(G))) {
         const dim3 grid((unsigned)((W + 31) / 32 * ((H + TH - 1) / TH) * B), (ci + BM - 1) / BM);
-        f<<<grid, 256, smem(G), st>>>(dy, w, dx, ci, co, Kp, B, H, W, add);
+        fdtd::launch_pdl_smem(f, grid, 256, smem(G), st, dy, w, dx, ci, co, Kp, B, H, W, add);
     } else {
         conv3<true>(dy, w, nullptr, dx, ci, co, (long long)B * H * W, H, W, add, 0, 1, nullptr, st);
     }
@@ -954,18 +1007,18 @@ int nn_conv3_wgrad(const float *dy, const float *x, float *gw, int ci, int co, i
     const int gx = (N + 127) / 128;
     if (W % 4 == 0 && aligned16(dy) && aligned16(x)) {
         if (co <= 32)
-            k_conv3_wgrad_t<2, 1><<<dim3(gx, 1, splits), 128, 0, st>>>(dy, x, gw, ci, co, B, H, W, kc, work);
+            fdtd::launch_pdl_smem(k_conv3_wgrad_t<2, 1>, dim3(gx, 1, splits), 128, 0, st, dy, x, gw, ci, co, B, H, W, kc, work);
         else if (co <= 48)
-            k_conv3_wgrad_t<3, 1><<<dim3(gx, 1, splits), 128, 0, st>>>(dy, x, gw, ci, co, B, H, W, kc, work);
+            fdtd::launch_pdl_smem(k_conv3_wgrad_t<3, 1>, dim3(gx, 1, splits), 128, 0, st, dy, x, gw, ci, co, B, H, W, kc, work);
         else
-            k_conv3_wgrad_t<3, 2><<<dim3(gx, (co + 95) / 96, splits), 256, 0, st>>>(dy, x, gw, ci, co, B, H, W, kc, work);
+            fdtd::launch_pdl_smem(k_conv3_wgrad_t<3, 2>, dim3(gx, (co + 95) / 96, splits), 256, 0, st, dy, x, gw, ci, co, B, H, W, kc, work);
     } else if (co <= 32)
-        k_conv3_wgrad<1, 2, 4><<<dim3(gx, 1, splits), 256, 0, st>>>(dy, x, gw, ci, co, P, H, W, kc, work);
+        fdtd::launch_pdl_smem(k_conv3_wgrad<1, 2, 4>, dim3(gx, 1, splits), 256, 0, st, dy, x, gw, ci, co, P, H, W, kc, work);
     else if (co <= 48)
-        k_conv3_wgrad<1, 3, 4><<<dim3(gx, 1, splits), 384, 0, st>>>(dy, x, gw, ci, co, P, H, W, kc, work);
+        fdtd::launch_pdl_smem(k_conv3_wgrad<1, 3, 4>, dim3(gx, 1, splits), 384, 0, st, dy, x, gw, ci, co, P, H, W, kc, work);
     else
-        k_conv3_wgrad<3, 2, 4><<<dim3(gx, (co + 95) / 96, splits), 256, 0, st>>>(dy, x, gw, ci, co, P, H, W, kc, work);
-    if (splits > 1) k_slices<<<slice_blocks((long long)co * N), 64, 0, st>>>(gw, work, (long long)co * N, splits);
+        fdtd::launch_pdl_smem(k_conv3_wgrad<3, 2, 4>, dim3(gx, (co + 95) / 96, splits), 256, 0, st, dy, x, gw, ci, co, P, H, W, kc, work);
+    if (splits > 1) fdtd::launch_pdl_smem(k_slices, slice_blocks((long long)co * N, 64), 64, 0, st, gw, work, (long long)co * N, splits);
     return status();
 }
 

@@ -15,6 +15,7 @@
 #include <stdint.h>
 
 #include "../../include/surrogate.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -39,6 +40,8 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, float alpha, 
                                               const float *__restrict__ B, int ldb, float beta, float *C, int ldc,
                                               int kc, float *part)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     __shared__ float As[GK][GT + 4];
     __shared__ float Bs[GK][GT + 4];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -99,6 +102,8 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, float alpha, 
 // C = sum over s = 0 .. S-1 of part[s] (in that order) + beta C.
 __global__ void k_splitk_sum(float *C, int ldc, const float *__restrict__ part, int M, int N, int S, float beta)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     const long long n = (long long)M * N;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         float acc = part[e];
@@ -113,6 +118,8 @@ __global__ void k_splitk_sum(float *C, int ldc, const float *__restrict__ part, 
 // arithmetic is done once, the nine stores of a warp are each contiguous.
 __global__ void k_im2col3(const float *x, int C, int B, int H, int W, float *col)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     const int HW = H * W;
     const long long P = (long long)B * HW, n = (long long)C * P;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -134,6 +141,8 @@ __global__ void k_im2col3(const float *x, int C, int B, int H, int W, float *col
 // that read it (gathered, so no atomics).
 __global__ void k_col2im3(const float *col, int C, int B, int H, int W, float *dx)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     const long long P = (long long)B * H * W, n = (long long)C * P;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(e / P);
@@ -153,6 +162,8 @@ __global__ void k_col2im3(const float *col, int C, int B, int H, int W, float *d
 
 __global__ void k_bias_act(float *y, const float *bias, int Cout, long long P, int relu)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     const long long n = (long long)Cout * P;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         float v = y[e] + bias[e / P];
@@ -166,6 +177,8 @@ __global__ void k_bias_act(float *y, const float *bias, int Cout, long long P, i
 __global__ void __launch_bounds__(1024) k_relu_bwd_bias(const float *y, float *dy, float *db, long long P, int relu,
                                                         int vec)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     __shared__ float part[32];
     const int c = blockIdx.x;
     float s = 0.0f;
@@ -212,6 +225,8 @@ __global__ void __launch_bounds__(1024) k_relu_bwd_bias(const float *y, float *d
 __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(128)
 k_relu_bwd_bias8(const float *__restrict__ y, float *dy, float *db, long long P, int relu)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     __shared__ float part[32];
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
@@ -253,6 +268,8 @@ k_relu_bwd_bias8(const float *__restrict__ y, float *dy, float *db, long long P,
 // 2 x 2 average pooling of planes [n][H][W] -> [n][H/2][W/2] and its adjoint.
 __global__ void k_pool2(const float *x, long long planes, int H, int W, float *y)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     const int h = H / 2, w = W / 2;
     const long long n = planes * h * w;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -265,6 +282,8 @@ __global__ void k_pool2(const float *x, long long planes, int H, int W, float *y
 
 __global__ void k_pool2_bwd(const float *dy, long long planes, int H, int W, float *dx)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     const long long n = planes * H * W;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         const long long pl = e / ((long long)H * W);
@@ -276,6 +295,8 @@ __global__ void k_pool2_bwd(const float *dy, long long planes, int H, int W, flo
 // 2x nearest upsampling of planes [n][h][w] -> [n][2h][2w] and its adjoint.
 __global__ void k_up2(const float *x, long long planes, int h, int w, float *y)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     const int H = 2 * h, W = 2 * w;
     const long long n = planes * H * W;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -287,6 +308,8 @@ __global__ void k_up2(const float *x, long long planes, int h, int w, float *y)
 
 __global__ void k_up2_bwd(const float *dy, long long planes, int h, int w, float *dx)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     const long long n = planes * h * w;
     const int W = 2 * w;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -314,6 +337,8 @@ __device__ __forceinline__ void each_pair(long long planes, int h, int w, F f)
 
 __global__ void k_pool2_v(const float4 *__restrict__ x, long long planes, int h, int w, float2 *y)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     each_pair(planes, h, w, [&](long long c, long long f, int w4) {
         const float4 a = x[f], b = x[f + w4];
         y[c] = make_float2(0.25f * (a.x + a.y + b.x + b.y), 0.25f * (a.z + a.w + b.z + b.w));
@@ -322,6 +347,8 @@ __global__ void k_pool2_v(const float4 *__restrict__ x, long long planes, int h,
 
 __global__ void k_pool2_bwd_v(const float2 *__restrict__ dy, long long planes, int h, int w, float4 *dx)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     each_pair(planes, h, w, [&](long long c, long long f, int w4) {
         const float2 g = dy[c];
         float4 a = dx[f], b = dx[f + w4];
@@ -340,6 +367,8 @@ __global__ void k_pool2_bwd_v(const float2 *__restrict__ dy, long long planes, i
 
 __global__ void k_up2_v(const float2 *__restrict__ x, long long planes, int h, int w, float4 *y)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     each_pair(planes, h, w, [&](long long c, long long f, int w4) {
         const float2 v = x[c];
         y[f] = y[f + w4] = make_float4(v.x, v.x, v.y, v.y);
@@ -348,6 +377,8 @@ __global__ void k_up2_v(const float2 *__restrict__ x, long long planes, int h, i
 
 __global__ void k_up2_bwd_v(const float4 *__restrict__ dy, long long planes, int h, int w, float2 *dx)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     each_pair(planes, h, w, [&](long long c, long long f, int w4) {
         const float4 a = dy[f], b = dy[f + w4];
         float2 v = dx[c];
@@ -366,6 +397,8 @@ bool pairs_ok(int w, const void *coarse, const void *fine)
 // dy = 2 (y - t) / n.
 __global__ void k_mse(const float *y, const float *t, long long n, float *dy, double *loss)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     double s = 0.0;
     const float inv = 2.0f / (float)n;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -393,6 +426,8 @@ struct AdamList {
 __global__ void __launch_bounds__(TPB) k_adam(const __grid_constant__ AdamList L, float lr, float b1, float b2, float eps,
                                               float c1, float c2)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     int i = 0, hi = L.count - 1;
     while (i < hi) {
         const int mid = (i + hi + 1) / 2;
@@ -418,6 +453,8 @@ __global__ void __launch_bounds__(TPB) k_adam(const __grid_constant__ AdamList L
 
 __global__ void k_zero_f(float *x, long long n)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
         x[e] = 0.0f;
 }
@@ -454,6 +491,8 @@ __global__ void __launch_bounds__(256) k_gemm_bf16(int M, int N, int K, float al
                                                    int lda, const float *__restrict__ B, int ldb, float beta,
                                                    float *C, int ldc, int kc, float *part)
 {
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
     __shared__ __align__(16) __nv_bfloat16 As[BM][BKP];
     __shared__ __align__(16) __nv_bfloat16 Bs[BN][BKP];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -572,11 +611,11 @@ int nn_gemm(int transA, int transB, int M, int N, int K, float alpha, const floa
     int kc = 0;
     const int splits = splitk(M, N, K, (long long)((N + GT - 1) / GT) * ((M + GT - 1) / GT), GK, work_elems, &kc);
     dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT, splits);
-    if (!transA && !transB) k_gemm<false, false><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
-    else if (!transA && transB) k_gemm<false, true><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
-    else if (transA && !transB) k_gemm<true, false><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
-    else k_gemm<true, true><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
-    if (splits > 1) k_splitk_sum<<<blocks_for((long long)M * N), TPB, 0, st>>>(C, ldc, work, M, N, splits, beta);
+    if (!transA && !transB) fdtd::launch_pdl_smem(k_gemm<false, false>, grid, 256, 0, st, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
+    else if (!transA && transB) fdtd::launch_pdl_smem(k_gemm<false, true>, grid, 256, 0, st, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
+    else if (transA && !transB) fdtd::launch_pdl_smem(k_gemm<true, false>, grid, 256, 0, st, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
+    else fdtd::launch_pdl_smem(k_gemm<true, true>, grid, 256, 0, st, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
+    if (splits > 1) fdtd::launch_pdl_smem(k_splitk_sum, blocks_for((long long)M * N), TPB, 0, st, C, ldc, work, M, N, splits, beta);
     return status(st);
 }
 
@@ -591,11 +630,11 @@ int nn_gemm_bf16(int transA, int transB, int M, int N, int K, float alpha, const
     int kc = 0;
     const int splits = splitk(M, N, K, (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM), BK, work_elems, &kc);
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, splits);
-    if (!transA && !transB) k_gemm_bf16<false, false><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
-    else if (!transA && transB) k_gemm_bf16<false, true><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
-    else if (transA && !transB) k_gemm_bf16<true, false><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
-    else k_gemm_bf16<true, true><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
-    if (splits > 1) k_splitk_sum<<<blocks_for((long long)M * N), TPB, 0, st>>>(C, ldc, work, M, N, splits, beta);
+    if (!transA && !transB) fdtd::launch_pdl_smem(k_gemm_bf16<false, false>, grid, 256, 0, st, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
+    else if (!transA && transB) fdtd::launch_pdl_smem(k_gemm_bf16<false, true>, grid, 256, 0, st, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
+    else if (transA && !transB) fdtd::launch_pdl_smem(k_gemm_bf16<true, false>, grid, 256, 0, st, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
+    else fdtd::launch_pdl_smem(k_gemm_bf16<true, true>, grid, 256, 0, st, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kc, work);
+    if (splits > 1) fdtd::launch_pdl_smem(k_splitk_sum, blocks_for((long long)M * N), TPB, 0, st, C, ldc, work, M, N, splits, beta);
     return status(st);
 }
 
@@ -603,7 +642,7 @@ int nn_im2col3(const float *x, int C, int B, int H, int W, float *col, void *str
 {
     if (!x || !col || C <= 0 || B <= 0 || H <= 0 || W <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
-    k_im2col3<<<blocks_for((long long)C * 9 * B * H * W), TPB, 0, st>>>(x, C, B, H, W, col);
+    fdtd::launch_pdl_smem(k_im2col3, blocks_for((long long)C * 9 * B * H * W), TPB, 0, st, x, C, B, H, W, col);
     return status(st);
 }
 
@@ -611,7 +650,7 @@ int nn_col2im3_add(const float *col, int C, int B, int H, int W, float *dx, void
 {
     if (!col || !dx || C <= 0 || B <= 0 || H <= 0 || W <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
-    k_col2im3<<<blocks_for((long long)C * B * H * W), TPB, 0, st>>>(col, C, B, H, W, dx);
+    fdtd::launch_pdl_smem(k_col2im3, blocks_for((long long)C * B * H * W), TPB, 0, st, col, C, B, H, W, dx);
     return status(st);
 }
 
@@ -619,7 +658,7 @@ int nn_bias_act(float *y, const float *bias, int Cout, long long P, int relu, vo
 {
     if (!y || !bias || Cout <= 0 || P <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
-    k_bias_act<<<blocks_for((long long)Cout * P), TPB, 0, st>>>(y, bias, Cout, P, relu);
+    fdtd::launch_pdl_smem(k_bias_act, blocks_for((long long)Cout * P), TPB, 0, st, y, bias, Cout, P, relu);
     return status(st);
 }
 
@@ -629,9 +668,9 @@ int nn_act_bwd_bias(const float *y, float *dy, float *db, int Cout, long long P,
     cudaStream_t st = (cudaStream_t)stream;
     const int vec = (P & 3) == 0 && (((uintptr_t)y | (uintptr_t)dy) & 15) == 0;
     if (vec && P >= 8 * 4096)  // eight values' loads in flight per thread; below, one block has them all at once
-        k_relu_bwd_bias8<<<8 * Cout, 128, 0, st>>>(y, dy, db, P, relu);
+        fdtd::launch_pdl_smem(k_relu_bwd_bias8, 8 * Cout, 128, 0, st, y, dy, db, P, relu);
     else
-        k_relu_bwd_bias<<<Cout, 1024, 0, st>>>(y, dy, db, P, relu, vec);
+        fdtd::launch_pdl_smem(k_relu_bwd_bias, Cout, 1024, 0, st, y, dy, db, P, relu, vec);
     return status(st);
 }
 
@@ -640,9 +679,9 @@ int nn_pool2(const float *x, long long planes, int H, int W, float *y, void *str
     if (!x || !y || planes <= 0 || H < 2 || W < 2 || (H | W) & 1) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     if (pairs_ok(W / 2, y, x))
-        k_pool2_v<<<blocks_for(planes * (H / 2) * (W / 4)), TPB, 0, st>>>((const float4 *)x, planes, H / 2, W / 2, (float2 *)y);
+        fdtd::launch_pdl_smem(k_pool2_v, blocks_for(planes * (H / 2) * (W / 4)), TPB, 0, st, (const float4 *)x, planes, H / 2, W / 2, (float2 *)y);
     else
-        k_pool2<<<blocks_for(planes * (H / 2) * (W / 2)), TPB, 0, st>>>(x, planes, H, W, y);
+        fdtd::launch_pdl_smem(k_pool2, blocks_for(planes * (H / 2) * (W / 2)), TPB, 0, st, x, planes, H, W, y);
     return status(st);
 }
 
@@ -651,9 +690,9 @@ int nn_pool2_bwd_add(const float *dy, long long planes, int H, int W, float *dx,
     if (!dy || !dx || planes <= 0 || H < 2 || W < 2 || (H | W) & 1) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     if (pairs_ok(W / 2, dy, dx))
-        k_pool2_bwd_v<<<blocks_for(planes * (H / 2) * (W / 4)), TPB, 0, st>>>((const float2 *)dy, planes, H / 2, W / 2, (float4 *)dx);
+        fdtd::launch_pdl_smem(k_pool2_bwd_v, blocks_for(planes * (H / 2) * (W / 4)), TPB, 0, st, (const float2 *)dy, planes, H / 2, W / 2, (float4 *)dx);
     else
-        k_pool2_bwd<<<blocks_for(planes * H * W), TPB, 0, st>>>(dy, planes, H, W, dx);
+        fdtd::launch_pdl_smem(k_pool2_bwd, blocks_for(planes * H * W), TPB, 0, st, dy, planes, H, W, dx);
     return status(st);
 }
 
@@ -662,9 +701,9 @@ int nn_up2(const float *x, long long planes, int h, int w, float *y, void *strea
     if (!x || !y || planes <= 0 || h <= 0 || w <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     if (pairs_ok(w, x, y))
-        k_up2_v<<<blocks_for(planes * h * (w / 2)), TPB, 0, st>>>((const float2 *)x, planes, h, w, (float4 *)y);
+        fdtd::launch_pdl_smem(k_up2_v, blocks_for(planes * h * (w / 2)), TPB, 0, st, (const float2 *)x, planes, h, w, (float4 *)y);
     else
-        k_up2<<<blocks_for(planes * 4 * h * w), TPB, 0, st>>>(x, planes, h, w, y);
+        fdtd::launch_pdl_smem(k_up2, blocks_for(planes * 4 * h * w), TPB, 0, st, x, planes, h, w, y);
     return status(st);
 }
 
@@ -673,9 +712,9 @@ int nn_up2_bwd_add(const float *dy, long long planes, int h, int w, float *dx, v
     if (!dy || !dx || planes <= 0 || h <= 0 || w <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     if (pairs_ok(w, dx, dy))
-        k_up2_bwd_v<<<blocks_for(planes * h * (w / 2)), TPB, 0, st>>>((const float4 *)dy, planes, h, w, (float2 *)dx);
+        fdtd::launch_pdl_smem(k_up2_bwd_v, blocks_for(planes * h * (w / 2)), TPB, 0, st, (const float4 *)dy, planes, h, w, (float2 *)dx);
     else
-        k_up2_bwd<<<blocks_for(planes * h * w), TPB, 0, st>>>(dy, planes, h, w, dx);
+        fdtd::launch_pdl_smem(k_up2_bwd, blocks_for(planes * h * w), TPB, 0, st, dy, planes, h, w, dx);
     return status(st);
 }
 
@@ -683,8 +722,8 @@ int nn_mse(const float *y, const float *t, long long n, float *dy, double *loss,
 {
     if (!y || !t || !dy || !loss || n <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
-    k_zero_f<<<1, 32, 0, st>>>((float *)loss, 2);
-    k_mse<<<blocks_for(n), TPB, 0, st>>>(y, t, n, dy, loss);
+    fdtd::launch_pdl_smem(k_zero_f, 1, 32, 0, st, (float *)loss, 2);
+    fdtd::launch_pdl_smem(k_mse, blocks_for(n), TPB, 0, st, y, t, n, dy, loss);
     return status(st);
 }
 
@@ -711,7 +750,7 @@ int nn_adam_multi(int count, float *const *p, const float *const *g, float *cons
             blocks += (int)(b < 152 * 16 ? b : 152 * 16);
         }
         L.first[L.count] = blocks;
-        k_adam<<<blocks, TPB, 0, st>>>(L, lr, beta1, beta2, eps, c1, c2);
+        fdtd::launch_pdl_smem(k_adam, blocks, TPB, 0, st, L, lr, beta1, beta2, eps, c1, c2);
     }
     return status(st);
 }
@@ -727,7 +766,7 @@ int nn_zero(float *x, long long n, void *stream)
     if (!x || n < 0) return 1;
     if (n == 0) return 0;
     cudaStream_t st = (cudaStream_t)stream;
-    k_zero_f<<<blocks_for(n), TPB, 0, st>>>(x, n);
+    fdtd::launch_pdl_smem(k_zero_f, blocks_for(n), TPB, 0, st, x, n);
     return status(st);
 }
 
