@@ -674,10 +674,10 @@ struct Ctx2D final : fdtd_ctx {
             // Measured, launch per step against blocked (us per forward /
             // full-history adjoint step): FP32 316^2 6.9 / 7.5 against 1.02 /
             // 1.28, 500^2 7.5 / 7.6 against 2.1 / 2.3, 1000^2 10.6 / 10.4
-            // against 4.9 / 6.2, 1400^2 13.1 / 15.3 against 8.0 / 10.4, 2048^2
-            // 23.2 / 25 against 17.3 / 22 (21.2 forward with the L2 window,
+            // against 4.5 / 6.1, 1400^2 13.1 / 15.3 against 6.9 / 10.5, 2048^2
+            // 23.2 / 25 against 13.2 / 19.6 (21.2 forward with the L2 window,
             // which the blocked launches do not take), 4096^2 77 / 86 against
-            // 69 / 86; FP64 160^2 12.1 / 15.1 against 3.3 / 3.3, 1000^2 52 /
+            // 47 / 69; FP64 160^2 12.1 / 15.1 against 3.3 / 3.3, 1000^2 52 /
             // 72 against 49 / 53.
             rt_auto = sizeof(R) == 4 || ncells <= 1LL << 20;
         }

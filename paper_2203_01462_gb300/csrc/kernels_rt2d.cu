@@ -77,8 +77,9 @@ constexpr int GAP_STAGED = 256;
 // per SM, and runs with the steps per launch set by the caller, have always
 // used 0, all others 1; both are kept, so that a design's results do not
 // change with the kernel that computes them.
-template <typename R, int MODE, int FORM>
-__global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
+// NB: blocks per SM the registers have to leave room for.
+template <typename R, int MODE, int FORM, int NB>
+__global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB)
     k_rt2d(const __grid_constant__ Geo2D g, const __grid_constant__ State2D<R> in,
            const __grid_constant__ State2D<R> out, int slot, const __grid_constant__ Pml1D<R> px,
            const __grid_constant__ Pml1D<R> py, const __grid_constant__ Rt2D<R> w)
@@ -152,8 +153,8 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
     // 600 of a launch's 1080 instructions per warp: 2048^2 22.5 -> 17.8 us per
     // forward step, 27 -> 23.5 per adjoint step, 1000^2 5.9 -> 4.9.  (Copying
     // the next tile's state into shared memory while one is stepped, in
-    // persistent blocks, gained nothing on top: 18.5; instruction issue, at
-    // half its rate, and the step's barrier are what is left.)
+    // persistent blocks, gained nothing on top: 18.5; a second block per SM
+    // did: 13.2, see launch_rt2d.)
     auto body = [&](auto vc, auto dc) {
     constexpr bool V = decltype(vc)::value, D = decltype(dc)::value, PL = V || D;
     // ---- load the region
@@ -654,8 +655,8 @@ __global__ void k_rt2d_coef(const __grid_constant__ Geo2D g, int slot, const R *
 
 // A wave's fixed part in row steps, fitted to FP32 halos of 4, 6, 8 on seven
 // grids (us per forward step, halo 4 / 6 / 8: 316^2 1.60 / 1.29 / 1.12, 530^2
-// 2.77 / 2.18 / 2.47, 700^2 3.47 / 3.14 / 3.33, 1400^2 8.2 / 7.9 / 9.0, 2048^2
-// 18.0 / 17.4 / 18.3: within 2 % of the best on each), and in FP64 from 3 us of
+// 2.77 / 2.18 / 2.47, 700^2 3.47 / 3.14 / 3.33, 1400^2 7.2 / 6.9 / 7.9, 2048^2
+// 13.7 / 13.2 / 14.1: within 2 % of the best on each), and in FP64 from 3 us of
 // launch against 0.24 us per row step.
 template <typename R>
 Rt2DPlan rt2d_plan(int nx, int ny, int sms, int steps)
@@ -665,34 +666,82 @@ Rt2DPlan rt2d_plan(int nx, int ny, int sms, int steps)
     return rt_tile_plan(nx, ny, sms, D::W, D::RPW, D::MAXW, !F64 && steps > 4 ? RT2D_MAX : 4, F64 ? 10.0 : 350.0);
 }
 
+template <typename R, int NB>
+bool allow(size_t b)
+{
+    return cudaFuncSetAttribute(k_rt2d<R, 0, 0, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) == cudaSuccess &&
+           cudaFuncSetAttribute(k_rt2d<R, 1, 0, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) == cudaSuccess &&
+           cudaFuncSetAttribute(k_rt2d<R, 0, 1, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) == cudaSuccess &&
+           cudaFuncSetAttribute(k_rt2d<R, 1, 1, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) == cudaSuccess;
+}
+
 template <typename R>
 bool rt2d_ready()
 {
     int dev = 0, smem = 0;
     const int Mx = Shape<R>::MAXW;
     const size_t b = std::max(smem_words<R>(Mx, RT2D_MAX, 0, 0), smem_words<R>(Mx, RT2D_MAX, GAP_STAGED, 1)) * sizeof(R);
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-        b > (size_t)smem ||
-        cudaFuncSetAttribute(k_rt2d<R, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) != cudaSuccess ||
-        cudaFuncSetAttribute(k_rt2d<R, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) != cudaSuccess ||
-        cudaFuncSetAttribute(k_rt2d<R, 0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) != cudaSuccess ||
-        cudaFuncSetAttribute(k_rt2d<R, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return true;
+    bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+              cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+              b <= (size_t)smem && allow<R, 1>(b);
+    if constexpr (sizeof(R) == 4) ok = ok && allow<R, 2>(b);
+    if (!ok) cudaGetLastError();
+    return ok;
 }
 
-template <typename R>
-int launch_rt2d(int mode, const Geo2D &g, const State2D<R> &in, const State2D<R> &out, int slot, const Pml1D<R> &px,
-                const Pml1D<R> &py, const Rt2D<R> &w, const Rt2DPlan &p, cudaStream_t st)
+template <typename R, int NB>
+void launch_nb(int mode, const Geo2D &g, const State2D<R> &in, const State2D<R> &out, int slot, const Pml1D<R> &px,
+               const Pml1D<R> &py, const Rt2D<R> &w, const Rt2DPlan &p, cudaStream_t st)
 {
     const int Mg = g.gnx * g.gny;
     const size_t smem = smem_words<R>(p.nw, w.count, mode == 1 && Mg <= GAP_STAGED ? Mg : 0, mode) * sizeof(R);
     const dim3 block(32, p.nw), grid(p.bx, p.by);
-    const auto k = mode == 0 ? (p.form ? k_rt2d<R, 0, 1> : k_rt2d<R, 0, 0>) : (p.form ? k_rt2d<R, 1, 1> : k_rt2d<R, 1, 0>);
+    const auto k = mode == 0 ? (p.form ? k_rt2d<R, 0, 1, NB> : k_rt2d<R, 0, 0, NB>)
+                             : (p.form ? k_rt2d<R, 1, 1, NB> : k_rt2d<R, 1, 0, NB>);
     launch_pdl_smem(k, grid, block, smem, st, g, in, out, slot, px, py, w);
+}
+
+// Tiles whose region is plain background (V; those of the source's rows counted too).
+template <typename R>
+int background_tiles(const Geo2D &g, const Rt2DPlan &p)
+{
+    using D = Shape<R>;
+    const int lo = std::max(g.npml, 1), H = p.halo, h = p.nw * D::RPW;
+    int cin = 0, cdes = 0, rin = 0, rdes = 0;
+    for (int b = 0; b < p.bx; ++b) {
+        const int x = b * p.tw - H;
+        if (x < lo || x + D::W - 1 > g.nx - 2 - lo) continue;
+        ++cin;
+        cdes += x < g.dxa + g.dp && x + D::W > g.dxa;
+    }
+    for (int b = 0; b < p.by; ++b) {
+        const int y = b * p.th - H;
+        if (y - 1 < lo || y + h - 1 > g.ny - 2 - lo) continue;
+        ++rin;
+        rdes += y < g.dy0 + g.dny && y + h > g.dy0;
+    }
+    return cin * rin - cdes * rdes;
+}
+
+// Two blocks per SM (64 registers a thread: the background's instance fits,
+// the others spill) once there are more than four waves: one block's loads and
+// stores then overlap the other's steps.  us per forward step, one and two
+// blocks per SM: 700^2 (3.2 waves) 3.13 / 3.15, 850^2 (4.8) 3.87 / 3.75, 1400^2
+// 8.0 / 6.9, 2048^2 17.8 / 13.2, 1500^2 nearly all design box 13.0 / 11.3.  The
+// adjoint, which spills 1.9 kB outside the background, takes it where five
+// eighths of the tiles are background: 2048^2 with a 1024^2 design box (66 %)
+// 22.3 / 19.6, 2200 x 1000 with 300^2 (80 %) 9.3 / 8.5, but 1200^2 with 600^2
+// (58 %) 8.3 / 8.9 and 1500^2 with 1400^2 (5 %) 20.1 / 22.5.
+template <typename R>
+int launch_rt2d(int mode, const Geo2D &g, const State2D<R> &in, const State2D<R> &out, int slot, const Pml1D<R> &px,
+                const Pml1D<R> &py, const Rt2D<R> &w, const Rt2DPlan &p, cudaStream_t st)
+{
+    if constexpr (sizeof(R) == 4)
+        if (p.bx * p.by > 4 * 152 && (mode == 0 || 8 * background_tiles<R>(g, p) >= 5 * p.bx * p.by)) {
+            launch_nb<R, 2>(mode, g, in, out, slot, px, py, w, p, st);
+            return 1;
+        }
+    launch_nb<R, 1>(mode, g, in, out, slot, px, py, w, p, st);
     return 1;
 }
 
