@@ -1003,11 +1003,15 @@ int nn_conv3_wgrad(const float *dy, const float *x, float *gw, int ci, int co, i
     const long long P = (long long)B * H * W;
     long long kc = 0;
     const int N = 9 * ci, splits = nn_splitk_bf16(co, N, P, work_elems, &kc);
-    // eight warps (twelve for 48 rows) on tiles of 32, 48 or 96 rows x 128 columns
+    // tiles of 32, 48 or 96 rows x 128 columns; the K slices make about two
+    // blocks per SM, so few rows take more warps with less each (32 rows: eight
+    // warps of 16 rows 3.45, four of 32 3.55 ms per 8 x 256^2 training step; 48
+    // rows as four of 48 or twelve of 16 the same, 96 as eight of 48 3.55, of
+    // 32 3.58)
     const int gx = (N + 127) / 128;
     if (W % 4 == 0 && aligned16(dy) && aligned16(x)) {
         if (co <= 32)
-            fdtd::launch_pdl_smem(k_conv3_wgrad_t<2, 1>, dim3(gx, 1, splits), 128, 0, st, dy, x, gw, ci, co, B, H, W, kc, work);
+            fdtd::launch_pdl_smem(k_conv3_wgrad_t<1, 2>, dim3(gx, 1, splits), 256, 0, st, dy, x, gw, ci, co, B, H, W, kc, work);
         else if (co <= 48)
             fdtd::launch_pdl_smem(k_conv3_wgrad_t<3, 1>, dim3(gx, 1, splits), 128, 0, st, dy, x, gw, ci, co, B, H, W, kc, work);
         else
