@@ -37,14 +37,13 @@ namespace {
 // Tiles: 8 x 8 x 2 threads, four x-adjacent nodes each, i.e.
 // 32 x 8 x 2 nodes (a warp reads 128 contiguous bytes per row).  Shapes
 // (at 768 threads per SM): 8x8x4 at 3 / 8x8x2 at 6 / 4x8x4 at 6 / 8x4x2 at
-// 12 per SM; 8x8x2 and 4x8x4 were fastest, by 3-5 %.  Blocks per SM in
-// FP32 (the register budget): H 6 (80 registers), forward E 7 (72), adjoint
-// E 6 (80).  With the CPML terms taken one axis at a time the kernels need
-// about 100 registers unbounded (128-136 with all six psi pairs held), so
-// these bounds spill little (16-44 B; 148 B in the adjoint E).  256^3
-// forward step: 5 blocks everywhere 242.6 us, 6 everywhere 229.3, H and
-// forward E at 7 227.4, everything at 7 227.4 (adjoint 465 against 457 at
-// 6), H at 7 with E at 6 231.7.
+// 12 per SM; 8x8x2 and 4x8x4 were fastest, by 3-5 %.  Blocks per SM in FP32
+// (the register budget): H and forward E 7 (72 registers), adjoint E 6 (80).
+// With the CPML terms taken one axis at a time the general path needs about
+// 100 registers unbounded, so these bounds spill (24 B, 128 B in the adjoint
+// E, 40 B in H).  256^3 forward / recompute + adjoint step, us, by blocks of
+// H / E / adjoint E: 6 / 7 / 6 219.1 / 442.5, 7 / 7 / 6 218.4 / 441.1, 8 / 7 / 6
+// 229.0 / 462.8, 6 / 8 / 6 227.7 / 451.4, 6 / 7 / 7 219.1 / 445.9.
 // FP64: one node per thread, blocks of one warp on 8 x 4 nodes.  There the
 // two FP64 units of an SM are the bound (16 cycles per instruction, whatever
 // lanes are active), and they should have even shares of full warps: tiles of
@@ -358,6 +357,46 @@ __device__ __forceinline__ void h_tile(const Geo3D &g, const State3D<R> &s, cons
     if (i0 >= n0 || j >= n1 || k >= n2) return;
     const long long q = k * g.PP + (long long)j * g.px + i0;
     const long long P = g.px, PP = g.PP;
+    if constexpr (N == 4 && !COH) {
+        // A tile clear of walls, absorbing layer and plane-wave faces (60 % of
+        // them at 256^3): straight code, the same bits.  With its twin in the
+        // E half step 225.5 -> 218.4 us per forward step, 453.7 -> 441.1 per
+        // recompute + adjoint step; 512 x 512 x 384 1211 -> 1180, 2492 -> 2414.
+        // (Instances for tiles with a y- or z-slab only gained nothing more.)
+        const int x0 = bx * SH::BX * N, y0 = by * SH::BY, z0 = bz * SH::BZ, np1 = g.npml + 1;
+        bool plain = x0 >= np1 && x0 + SH::BX * N <= n0 - np1 && y0 >= np1 && y0 + SH::BY <= n1 - np1 && z0 >= np1 &&
+                     z0 + SH::BZ <= n2 - np1;
+        if (FOLD) {
+            auto has = [](int lo, int n, int p) { return (unsigned)(p - lo) < (unsigned)n; };
+            plain &= !(has(z0, SH::BZ, g.tf_lo[2] - 1) || has(z0, SH::BZ, g.tf_hi[2]) || has(y0, SH::BY, g.tf_lo[1] - 1) ||
+                       has(y0, SH::BY, g.tf_hi[1]));
+        }
+        if (plain) {
+            R ex[N], exN[N], exU[N], ey[N], eyU[N], ez[N], ezN[N], hx[N], hy[N], hz[N];
+            ld4(s.E[0] + q, ex);
+            ld4(s.E[1] + q, ey);
+            ld4(s.E[2] + q, ez);
+            ld4(s.E[0] + q + P, exN);
+            ld4(s.E[2] + q + P, ezN);
+            ld4(s.E[0] + q + PP, exU);
+            ld4(s.E[1] + q + PP, eyU);
+            ld4(s.H[0] + q, hx);
+            ld4(s.H[1] + q, hy);
+            ld4(s.H[2] + q, hz);
+            const R eyE = s.E[1][q + N], ezE = s.E[2][q + N], S = c.S;
+#pragma unroll
+            for (int v = 0; v < N; ++v) {
+                const R ezx = v < N - 1 ? ez[v < N - 1 ? v + 1 : v] : ezE, eyx = v < N - 1 ? ey[v < N - 1 ? v + 1 : v] : eyE;
+                hx[v] = rn_sub(hx[v], rn_mul(S, (ezN[v] - ez[v]) - (eyU[v] - ey[v])));
+                hy[v] = rn_sub(hy[v], rn_mul(S, (exU[v] - ex[v]) - (ezx - ez[v])));
+                hz[v] = rn_sub(hz[v], rn_mul(S, (eyx - ey[v]) - (exN[v] - ex[v])));
+            }
+            st4(s.H[0] + q, hx);
+            st4(s.H[1] + q, hy);
+            st4(s.H[2] + q, hz);
+            return;
+        }
+    }
     const bool yin = j <= n1 - 2, zin = k <= n2 - 2, xin = i0 + N <= n0 - 1;  // next row / plane / node exist
     const int np = g.npml;
     const int sy = slabH(j, n1, np), sz = slabH(k, n2, np);
@@ -460,7 +499,7 @@ __device__ __forceinline__ void h_tile(const Geo3D &g, const State3D<R> &s, cons
 // The H half step of the whole grid, bottom up or (zrev) top down; FOLD:
 // with the plane wave's H-face corrections of incident row inc.
 template <typename R, bool FOLD>
-__global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(R) == 4 ? 6 : 24)
+__global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(R) == 4 ? 7 : 24)
     k_h3d(Geo3D g, State3D<R> s, int slot, Pml3D<R> pm, int zrev, const R *inc)
 {
     wait_previous_grid();
@@ -485,6 +524,45 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
     if (i0 >= n0 || j >= n1 || k >= n2) return;
     const long long q = k * g.PP + (long long)j * g.px + i0;
     const long long P = g.px, PP = g.PP;
+    const bool touches = (x0 < g.d0[0] + g.dn[0] && x0 + TX > g.d0[0] && y0 < g.d0[1] + g.dn[1] &&
+                          y0 + TY > g.d0[1] && z0 < g.d0[2] + g.dn[2] && z0 + TZ > g.d0[2]) ||
+                         (MODE == 0 && x0 < g.s1[0] && x0 + TX > g.s0[0] && y0 < g.s1[1] && y0 + TY > g.s0[1] &&
+                          z0 < g.s1[2] && z0 + TZ > g.s0[2]);
+    if constexpr (N == 4 && !COH) {
+        // a tile clear of walls, absorbing layer, design box, source and plane-wave faces
+        const int np1 = g.npml + 1;
+        bool plain = !touches && x0 >= np1 && x0 + TX <= n0 - np1 && y0 >= np1 && y0 + TY <= n1 - np1 && z0 >= np1 &&
+                     z0 + TZ <= n2 - np1;
+        if (FOLD && MODE == 0) {
+            auto has = [](int lo, int n, int p) { return (unsigned)(p - lo) < (unsigned)n; };
+            plain &= !(has(z0, TZ, g.tf_lo[2]) || has(z0, TZ, g.tf_hi[2]) || has(x0, TX, g.tf_lo[0]) || has(x0, TX, g.tf_hi[0]));
+        }
+        if (plain) {
+            R hx[N], hxS[N], hxD[N], hy[N], hyD[N], hz[N], hzS[N], ex[N], ey[N], ez[N];
+            ld4(s.H[0] + q, hx);
+            ld4(s.H[1] + q, hy);
+            ld4(s.H[2] + q, hz);
+            ld4(s.H[0] + q - P, hxS);
+            ld4(s.H[2] + q - P, hzS);
+            ld4(s.H[0] + q - PP, hxD);
+            ld4(s.H[1] + q - PP, hyD);
+            ld4(s.E[0] + q, ex);
+            ld4(s.E[1] + q, ey);
+            ld4(s.E[2] + q, ez);
+            const R hyW = s.H[1][q - 1], hzW = s.H[2][q - 1], f = rcp(k < g.sub_hi ? c.eps_sub : c.eps_s);
+#pragma unroll
+            for (int v = 0; v < N; ++v) {
+                const R hyx = v > 0 ? hy[v > 0 ? v - 1 : 0] : hyW, hzx = v > 0 ? hz[v > 0 ? v - 1 : 0] : hzW;
+                ex[v] = rn_fma(rn_mul(c.S, (hz[v] - hzS[v]) - (hy[v] - hyD[v])), f, ex[v]);
+                ey[v] = rn_fma(rn_mul(c.S, (hx[v] - hxD[v]) - (hz[v] - hzx)), f, ey[v]);
+                ez[v] = rn_fma(rn_mul(c.S, (hy[v] - hyx) - (hx[v] - hxS[v])), f, ez[v]);
+            }
+            st4(s.E[0] + q, ex);
+            st4(s.E[1] + q, ey);
+            st4(s.E[2] + q, ez);
+            return;
+        }
+    }
     const int np = g.npml;
     const int sy = slabE(j, n1, np), sz = slabE(k, n2, np);
     const bool xslab = i0 < np || i0 + N - 1 >= n0 - np;
@@ -553,10 +631,6 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
         if (cc == 1) return j <= n1 - 2 && imid && kmid;
         return k <= n2 - 2 && imid && jmid;
     };
-    const bool touches = (x0 < g.d0[0] + g.dn[0] && x0 + TX > g.d0[0] && y0 < g.d0[1] + g.dn[1] &&
-                          y0 + TY > g.d0[1] && z0 < g.d0[2] + g.dn[2] && z0 + TZ > g.d0[2]) ||
-                         (MODE == 0 && x0 < g.s1[0] && x0 + TX > g.s0[0] && y0 < g.s1[1] && y0 + TY > g.s0[1] &&
-                          z0 < g.s1[2] && z0 + TZ > g.s0[2]);
     // (FP64 reciprocals, some fifteen operations, come from the host; FP32's
     // are rounded from FP32 operands)
     constexpr bool F64 = sizeof(R) == 8;
