@@ -230,6 +230,7 @@ k_relu_bwd_bias8(const float *__restrict__ y, float *dy, float *db, long long P,
     __shared__ float part[32];
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
+    cl.barrier_arrive();
     const int rank = blockIdx.x & 7, c = blockIdx.x >> 3, warp = rank * 4 + (threadIdx.x >> 5);
     const float4 *y4 = reinterpret_cast<const float4 *>(y + (long long)c * P);
     float4 *d4 = reinterpret_cast<float4 *>(dy + (long long)c * P);
@@ -256,6 +257,7 @@ k_relu_bwd_bias8(const float *__restrict__ y, float *dy, float *db, long long P,
             }
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    cl.barrier_wait();  // the first block has started: its shared memory can be written
     if ((threadIdx.x & 31) == 0) *cl.map_shared_rank(part + warp, 0) = s;
     cl.sync();
     if (rank == 0 && threadIdx.x < 32) {
