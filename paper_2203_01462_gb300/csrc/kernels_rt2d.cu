@@ -77,9 +77,10 @@ constexpr int GAP_STAGED = 256;
 // per SM, and runs with the steps per launch set by the caller, have always
 // used 0, all others 1; both are kept, so that a design's results do not
 // change with the kernel that computes them.
-// NB: blocks per SM the registers have to leave room for.
+// NB: blocks per SM the registers have to leave room for; 0: one, and only
+// the general kind of region (see launch_rt2d).
 template <typename R, int MODE, int FORM, int NB>
-__global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB)
+__global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
     k_rt2d(const __grid_constant__ Geo2D g, const __grid_constant__ State2D<R> in,
            const __grid_constant__ State2D<R> out, int slot, const __grid_constant__ Pml1D<R> px,
            const __grid_constant__ Pml1D<R> py, const __grid_constant__ Rt2D<R> w)
@@ -608,15 +609,19 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB)
         }
     }
     };
-    const int lo = max(np, 1), xe = xr + W - 1, ye = yr + nw * RPW - 1;
-    const bool inner = xr >= lo && xe <= nx - 2 - lo && yr - 1 >= lo && ye <= ny - 2 - lo &&
-                       !(xr < g.gx0 + g.gnx && xe >= g.gx0 && yr < g.gy0 + g.gny && ye >= g.gy0) &&
-                       !(MODE == 0 && xr < g.sx1 && xe >= g.sx0 && yr < g.sy1 && ye >= g.sy0);
-    const bool invac = xr >= g.dxa + g.dp || xe < g.dxa || yr >= g.dy0 + g.dny || ye < g.dy0;
-    const bool indes = xr >= g.dx0 && xe < g.dx0 + g.dnx && yr >= g.dy0 && ye < g.dy0 + g.dny;
-    if (inner && invac) body(std::true_type{}, std::false_type{});
-    else if (inner && indes) body(std::false_type{}, std::true_type{});
-    else body(std::false_type{}, std::false_type{});
+    if constexpr (NB == 0) {
+        body(std::false_type{}, std::false_type{});
+    } else {
+        const int lo = max(np, 1), xe = xr + W - 1, ye = yr + nw * RPW - 1;
+        const bool inner = xr >= lo && xe <= nx - 2 - lo && yr - 1 >= lo && ye <= ny - 2 - lo &&
+                           !(xr < g.gx0 + g.gnx && xe >= g.gx0 && yr < g.gy0 + g.gny && ye >= g.gy0) &&
+                           !(MODE == 0 && xr < g.sx1 && xe >= g.sx0 && yr < g.sy1 && ye >= g.sy0);
+        const bool invac = xr >= g.dxa + g.dp || xe < g.dxa || yr >= g.dy0 + g.dny || ye < g.dy0;
+        const bool indes = xr >= g.dx0 && xe < g.dx0 + g.dnx && yr >= g.dy0 && ye < g.dy0 + g.dny;
+        if (inner && invac) body(std::true_type{}, std::false_type{});
+        else if (inner && indes) body(std::false_type{}, std::true_type{});
+        else body(std::false_type{}, std::false_type{});
+    }
 }
 
 // The Drude coefficients of the pitched design box, in the operations of
@@ -684,7 +689,7 @@ bool rt2d_ready()
     bool ok = cudaGetDevice(&dev) == cudaSuccess &&
               cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
               b <= (size_t)smem && allow<R, 1>(b);
-    if constexpr (sizeof(R) == 4) ok = ok && allow<R, 2>(b);
+    if constexpr (sizeof(R) == 4) ok = ok && allow<R, 2>(b) && allow<R, 0>(b);
     if (!ok) cudaGetLastError();
     return ok;
 }
@@ -723,6 +728,9 @@ int background_tiles(const Geo2D &g, const Rt2DPlan &p)
     return cin * rin - cdes * rdes;
 }
 
+// One wave of tiles: it ends with its slowest tile, which is a general one, and
+// that one is faster alone (316^2 1.03 / 1.30 us per forward / adjoint step, with
+// the instances for background and design box beside it 1.10 / 1.36).
 // Two blocks per SM (64 registers a thread: the background's instance fits,
 // the others spill) once there are more than four waves: one block's loads and
 // stores then overlap the other's steps.  us per forward step, one and two
@@ -736,11 +744,16 @@ template <typename R>
 int launch_rt2d(int mode, const Geo2D &g, const State2D<R> &in, const State2D<R> &out, int slot, const Pml1D<R> &px,
                 const Pml1D<R> &py, const Rt2D<R> &w, const Rt2DPlan &p, cudaStream_t st)
 {
-    if constexpr (sizeof(R) == 4)
+    if constexpr (sizeof(R) == 4) {
+        if (p.bx * p.by <= 152) {
+            launch_nb<R, 0>(mode, g, in, out, slot, px, py, w, p, st);
+            return 1;
+        }
         if (p.bx * p.by > 4 * 152 && (mode == 0 || 8 * background_tiles<R>(g, p) >= 5 * p.bx * p.by)) {
             launch_nb<R, 2>(mode, g, in, out, slot, px, py, w, p, st);
             return 1;
         }
+    }
     launch_nb<R, 1>(mode, g, in, out, slot, px, py, w, p, st);
     return 1;
 }
