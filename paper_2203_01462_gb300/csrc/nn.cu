@@ -408,8 +408,15 @@ __global__ void k_mse(const float *y, const float *t, long long n, float *dy, do
         dy[e] = inv * d;
         s += (double)d * (double)d;
     }
+    // one atomic per block: one per warp made 16384 of them on one address for 2 MB (30 us; 8 so)
+    __shared__ double part[TPB / 32];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, s / (double)n);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < TPB / 32; ++q) s += part[q];
+        atomicAdd(loss, s / (double)n);
+    }
 }
 
 // Adam on up to ADAM_T tensors in one launch: blocks of ADAM_E elements, the
@@ -572,6 +579,34 @@ __global__ void __launch_bounds__(256) k_gemm_bf16(int M, int N, int K, float al
             }
 }
 
+// K = 1: C[m][n] = alpha a[m] b[n] + beta C[m][n], four columns per thread, OUTER_M rows per block.
+constexpr int OUTER_M = 8;
+__global__ void __launch_bounds__(TPB) k_outer_bf16(int M, int N, float alpha, const float *__restrict__ A, int as,
+                                                    const float *__restrict__ B, float beta, float *C, int ldc)
+{
+    fdtd::pdl_wait();
+    fdtd::pdl_trigger();
+    const int n = (blockIdx.x * TPB + threadIdx.x) * 4, m0 = blockIdx.y * OUTER_M;
+    if (n >= N) return;
+    auto bf = [](float v) { return __bfloat162float(__float2bfloat16_rn(v)); };
+    const float4 b = *reinterpret_cast<const float4 *>(B + n);
+    const float bv[4] = {bf(b.x), bf(b.y), bf(b.z), bf(b.w)};
+    float4 old[OUTER_M];
+#pragma unroll
+    for (int i = 0; i < OUTER_M; ++i)
+        if (beta != 0.0f && m0 + i < M) old[i] = *reinterpret_cast<const float4 *>(C + (long long)(m0 + i) * ldc + n);
+#pragma unroll
+    for (int i = 0; i < OUTER_M; ++i) {
+        if (m0 + i >= M) break;
+        const float a = bf(A[(long long)(m0 + i) * as]);
+        const float c[4] = {old[i].x, old[i].y, old[i].z, old[i].w};
+        float o[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) o[v] = alpha * (a * bv[v]) + (beta != 0.0f ? beta * c[v] : 0.0f);
+        *reinterpret_cast<float4 *>(C + (long long)(m0 + i) * ldc + n) = make_float4(o[0], o[1], o[2], o[3]);
+    }
+}
+
 }  // namespace
 
 extern "C" {
@@ -629,6 +664,14 @@ int nn_gemm_bf16(int transA, int transB, int M, int N, int K, float alpha, const
     if (M == 0 || N == 0) return 0;
     if (K == 0) return nn_gemm(transA, transB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, work, work_elems, stream);
     cudaStream_t st = (cudaStream_t)stream;
+    if (K == 1 && !transB && N % 4 == 0 && ldc % 4 == 0 && (((uintptr_t)B | (uintptr_t)C) & 15) == 0 &&
+        M <= 65535 * OUTER_M) {
+        // nothing to sum: the tiles of k_gemm_bf16 would be one thirty-second full
+        // (input gradient of the 1 x 1 head, 24 x 524288: 68 us, 15 so)
+        fdtd::launch_pdl_smem(k_outer_bf16, dim3((N / 4 + TPB - 1) / TPB, (M + OUTER_M - 1) / OUTER_M), TPB, 0, st, M, N,
+                              alpha, A, transA ? 1 : lda, B, beta, C, ldc);
+        return status(st);
+    }
     int kc = 0;
     const int splits = splitk(M, N, K, (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM), BK, work_elems, &kc);
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, splits);
@@ -725,7 +768,7 @@ int nn_mse(const float *y, const float *t, long long n, float *dy, double *loss,
     if (!y || !t || !dy || !loss || n <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     fdtd::launch_pdl_smem(k_zero_f, 1, 32, 0, st, (float *)loss, 2);
-    fdtd::launch_pdl_smem(k_mse, blocks_for(n), TPB, 0, st, y, t, n, dy, loss);
+    fdtd::launch_pdl_smem(k_mse, blocks_for(n, 2 * 152), TPB, 0, st, y, t, n, dy, loss);
     return status(st);
 }
 

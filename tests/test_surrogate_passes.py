@@ -83,3 +83,24 @@ def test_adam_on_several_tensors_is_adam_on_each(count):
         assert all(torch.equal(s, t) for s, t in zip(a, b))
     arr[2][count - 1] = None  # a missing moment buffer is refused before anything is launched
     assert L.nn_adam_multi(count, *arr, (C.c_longlong * count)(*sizes), 1e-3, 0.9, 0.999, 1e-8, 3, None) == 1
+
+
+@pytest.mark.parametrize("ta", [0, 1])
+@pytest.mark.parametrize("M,N,beta,shift", [(1, 4, 0.0, 0), (8, 1024, 1.0, 0), (9, 1028, 0.5, 0), (24, 4096, 1.0, 0),
+                                            (24, 4095, 1.0, 0), (5, 64, 1.0, 1)])
+def test_gemm_bf16_of_depth_one(ta, M, N, beta, shift):
+    """One product per entry, exact in FP32; alpha = 1, and beta C + product
+    rounded once or twice: one unit in the last place of the larger term.
+    shift: operands that start 4 bytes past an aligned address."""
+    import torch
+    L = _lib()
+    g = torch.Generator(device="cuda").manual_seed(M * N)
+    A = torch.randn(M, generator=g, device="cuda")
+    B = torch.randn(N + shift, generator=g, device="cuda")[shift:]
+    Cm = torch.randn(M * N + shift, generator=g, device="cuda")[shift:].view(M, N)
+    prod = A.bfloat16().double()[:, None] * B.bfloat16().double()[None]
+    ref = prod + beta * Cm.double()
+    bound = 2.0 ** -23 * (prod.abs() + (beta * Cm.double()).abs())
+    assert L.nn_gemm_bf16(ta, 0, M, N, 1, 1.0, _p(A), M if ta else 1, _p(B), N, beta, _p(Cm), N, None, 0, None) == 0
+    torch.cuda.synchronize()
+    assert bool(((Cm.double() - ref).abs() <= bound).all())
