@@ -840,6 +840,7 @@ struct Ctx2D final : fdtd_ctx {
                 w.gap = Mg ? gap_hist : nullptr;
                 w.rec = base;
                 w.G = G;
+                w.ps = pair_scale(cfg.src_amp);
                 launches += launch_rt2d<R>(1, geo, A[curA], A[curA ^ 1], coef_slot, px, py, w, pl, stream);
                 curA ^= 1;
                 m -= w.count;
@@ -1371,7 +1372,7 @@ struct CtxP final : fdtd_ctx {
                 }
                 launches += launch_rt2dp_sens<R>(geo, coef_slot, rt_coef, Mdi_all(), arec,
                                                  rec + (size_t)(c_hi - 1 - slot0) * Mdi_all(), c_hi - c_lo, jsens, eprev, G,
-                                                 stream);
+                                                 pair_scale(cfg.src_amp), stream);
                 c_hi = c_lo;
             }
             cell_updates += (long long)(m_hi - m_lo) * ncells;

@@ -2,6 +2,8 @@
 // the kernel translation units.  Nothing here crosses the C ABI.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -265,6 +267,24 @@ template <typename R>
 int launch_step3d(int mode, const Geo3D &g, const State3D<R> &s, int coef_slot, const Pml3D<R> &pm,
                   const Step3D<R> &a, cudaStream_t st);
 
+// Scale of the products that a launch sums in FP32 pairs (rt_common.cuh), and
+// its inverse.  At amplitude 1 the products reach about 1: 2^100 leaves 20
+// binades up to the pair's limit.  They rise with the amplitude's square, so
+// past 2^8 the scale falls with it (down to 1), keeping a strong source's
+// largest products some four binades below the limit; a lower scale would
+// send more of a wave front's tail to FP64 (316^2-like grid, amplitude 1e4:
+// 2.8 us per step at 2^74).
+struct PairScale {
+    float up;
+    double down;
+};
+inline PairScale pair_scale(double src_amp)
+{
+    int e = 100;
+    if (std::isfinite(src_amp) && std::fabs(src_amp) > 1.0) e = std::min(e, std::max(0, 116 - 2 * std::ilogb(src_amp)));
+    return PairScale{std::ldexp(1.0f, e), std::ldexp(1.0, -e)};
+}
+
 // Temporally blocked 2D E_z steps with the tile in registers
 // (kernels_rt2d.cu): a block owns tw x th nodes with a halo and advances
 // count <= halo <= RT2D_MAX steps, reading state `in` and writing its tile
@@ -286,6 +306,7 @@ struct Rt2D {
     R *rec;
     const R *coef;
     double *G;
+    PairScale ps;   // adjoint, FP32
 };
 // Halo, tile sides, warps per block, blocks along x and y, and the rounding
 // form of the Drude update (kernels_rt2d.cu, FORM).
@@ -327,7 +348,7 @@ constexpr int RT2DP_CHUNK = 32;
 // adjoint J and E from one call to the next.
 template <typename R>
 int launch_rt2dp_sens(const GeoP &g, int coef_slot, const R *const coef[2], long long step, const R *ae, const R *fe,
-                      int count, R *const jsens[2], R *const eprev[2], double *const G[2], cudaStream_t st);
+                      int count, R *const jsens[2], R *const eprev[2], double *const G[2], PairScale ps, cudaStream_t st);
 template <typename R>
 Rt2DPlan rt2dp_plan(int nx, int ny, int sms);
 template <typename R>

@@ -506,13 +506,13 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
 #pragma unroll
                     for (int r = 0; r < RPW; ++r)
 #pragma unroll
-                        for (int v = 0; v < VX; ++v) far |= Pair::far(em[r][v], term[r][v] * Pair::SCALE);
+                        for (int v = 0; v < VX; ++v) far |= Pair::far(em[r][v], term[r][v] * w.ps.up);
                     if (__any_sync(0xffffffffu, far)) {
 #pragma unroll
                         for (int r = 0; r < RPW; ++r)
 #pragma unroll
                             for (int v = 0; v < VX; ++v)
-                                if (Pair::far(em[r][v], term[r][v] * Pair::SCALE)) {
+                                if (Pair::far(em[r][v], term[r][v] * w.ps.up)) {
                                     if (sens >> (r * VX + v) & 1u)
                                         w.G[d[r] + v] += (double)em[r][v] * (double)term[r][v];
                                     term[r][v] = R(0);
@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
 #pragma unroll
                     for (int r = 0; r < RPW; ++r)
 #pragma unroll
-                        for (int v = 0; v < VX; ++v) gp[r][v].add(em[r][v], term[r][v] * Pair::SCALE);
+                        for (int v = 0; v < VX; ++v) gp[r][v].add(em[r][v], term[r][v] * w.ps.up);
                 }
             }
 #pragma unroll
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
                 for (int v = 0; v < VX; ++v) {
                     if (!(sens >> (r * VX + v) & 1u)) continue;
                     if constexpr (F64) w.G[d[r] + v] = G[r][v];
-                    else w.G[d[r] + v] += gp[r][v].value();
+                    else w.G[d[r] + v] += gp[r][v].value(w.ps.down);
                 }
             }
         }

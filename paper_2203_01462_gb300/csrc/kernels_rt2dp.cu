@@ -438,7 +438,7 @@ template <typename R>
 __global__ void __launch_bounds__(128) k_rt2dp_sens(int slot, long long M0, long long M1, const R *__restrict__ coef0,
                                                     const R *__restrict__ coef1, long long step,
                                                     const R *__restrict__ ae, const R *__restrict__ fe, int count,
-                                                    R *j0, R *j1, R *e0, R *e1, double *G0, double *G1)
+                                                    R *j0, R *j1, R *e0, R *e1, double *G0, double *G1, PairScale ps)
 {
     constexpr int V = 16 / sizeof(R), U = 8;
     const Coef<R> &c = coef_at<R>(slot);
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(128) k_rt2dp_sens(int slot, long long M0, long
                     en[k][v] = R(0);
                 }
                 if constexpr (sizeof(R) == 8) g[v] += em[k][v] * en[k][v];
-                else far |= Pair::far(em[k][v], en[k][v] * Pair::SCALE);
+                else far |= Pair::far(em[k][v], en[k][v] * ps.up);
             }
         if constexpr (sizeof(R) == 4) {
             // a uniform branch: as selects, the FP64 operations would run for
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(128) k_rt2dp_sens(int slot, long long M0, long
                 for (int k = 0; k < U; ++k)
 #pragma unroll
                     for (int v = 0; v < V; ++v)
-                        if (Pair::far(em[k][v], en[k][v] * Pair::SCALE)) {
+                        if (Pair::far(em[k][v], en[k][v] * ps.up)) {
                             g[v] += (double)em[k][v] * (double)en[k][v];
                             en[k][v] = 0.0f;
                         }
@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(128) k_rt2dp_sens(int slot, long long M0, long
 #pragma unroll
             for (int k = 0; k < U; ++k)
 #pragma unroll
-                for (int v = 0; v < V; ++v) gp[v].add(em[k][v], en[k][v] * Pair::SCALE);
+                for (int v = 0; v < V; ++v) gp[v].add(em[k][v], en[k][v] * ps.up);
         }
     }
     if (!inside) return;
@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(128) k_rt2dp_sens(int slot, long long M0, long
     st16(jp, jo);
 #pragma unroll
     for (int v = 0; v < V; ++v)
-        if (bj[v] != R(0)) Gp[v] += g[v] + gp[v].value();  // not in the gap or the row padding
+        if (bj[v] != R(0)) Gp[v] += g[v] + gp[v].value(ps.down);  // not in the gap or the row padding
 }
 
 // The Drude coefficients of one component's pitched design edges, in the
@@ -601,12 +601,13 @@ int launch_rt2dp_coef(const GeoP &g, int slot, const R *const rho_t[2], R *const
 
 template <typename R>
 int launch_rt2dp_sens(const GeoP &g, int slot, const R *const coef[2], long long step, const R *ae, const R *fe, int count,
-                      R *const jsens[2], R *const eprev[2], double *const G[2], cudaStream_t st)
+                      R *const jsens[2], R *const eprev[2], double *const G[2], PairScale ps, cudaStream_t st)
 {
     constexpr int V = 16 / sizeof(R);
     const long long n = g.Mdi[0] + g.Mdi[1];
     launch_pdl(k_rt2dp_sens<R>, dim3((unsigned)((n + 128 * V - 1) / (128 * V))), dim3(128), st, slot, (long long)g.Mdi[0],
-               (long long)g.Mdi[1], coef[0], coef[1], step, ae, fe, count, jsens[0], jsens[1], eprev[0], eprev[1], G[0], G[1]);
+               (long long)g.Mdi[1], coef[0], coef[1], step, ae, fe, count, jsens[0], jsens[1], eprev[0], eprev[1], G[0], G[1],
+               ps);
     return 1;
 }
 
@@ -622,7 +623,7 @@ cudaError_t upload_coef_rt2dp(int slot, const Coef<R> &c, cudaStream_t st)
     template int launch_rt2dp<R>(int, const GeoP &, const StateP<R> &, const StateP<R> &, int, const PmlP<R> &,    \
                                  const RtP<R> &, const Rt2DPlan &, cudaStream_t);                                  \
     template int launch_rt2dp_sens<R>(const GeoP &, int, const R *const[2], long long, const R *, const R *, int,  \
-                                      R *const[2], R *const[2], double *const[2], cudaStream_t);                   \
+                                      R *const[2], R *const[2], double *const[2], PairScale, cudaStream_t);                   \
     template int launch_rt2dp_coef<R>(const GeoP &, int, const R *const[2], R *const[2], cudaStream_t);            \
     template cudaError_t upload_coef_rt2dp<R>(int, const Coef<R> &, cudaStream_t);
 RT2DP_INST(float)

@@ -64,24 +64,35 @@ __device__ __forceinline__ void cp8(void *s, const void *g)
                  : "memory");
 }
 
-// Exact sum of a few FP32 products as an unevaluated FP32 pair (hi + lo):
-// the adjoint's sensitivity sum of one launch.  A GB300 runs FP64 (and
-// conversions to it) at 1/64 of the FP32 rate, so one FP64 product and sum
-// per node and step (0.7 of 2.3 us per 316^2 adjoint step) becomes twelve
-// FP32 operations, and one FP64 addition per node and launch.  The product's
-// rounding error is recovered by an FMA and the sum's by Knuth's two-sum.
-// One factor is scaled by SCALE (exact), so that the tails of a wave front
-// (1e-30 and below) stay within FP32's range; value() undoes it.
+// Sum of the FP32 products of one launch (or chunk of launches) as an
+// unevaluated FP32 pair (hi + lo): a node's share of the adjoint's sensitivity,
+// which then goes into its FP64 accumulator.  A GB300 runs FP64 (and
+// conversions to it) at 1/64 of the FP32 rate, so one FP64 product and sum per
+// node and step (0.7 of 2.3 us per 316^2 adjoint step) becomes twelve FP32
+// operations, and one FP64 addition per node and launch.  The product's
+// rounding error is recovered by an FMA and the sum's by Knuth's two-sum; both
+// join lo, which is rounded, so a launch's sum is good to about 2^-47 of its
+// terms' magnitude.
+//
+// One factor is scaled by a power of two (PairScale; at least 1, so the scaling
+// loses nothing), which keeps the tails of a wave front (1e-30 and below, at
+// amplitude 1) within FP32's range; value() undoes it.  The products go with
+// the square of the source's amplitude, and so does the scale (pair_scale),
+// so that a strong source's products stay clear of FAR like a weak one's.
 struct Pair {
     float hi, lo;
-    static constexpr float SCALE = 0x1p100f;
-    // The product a (b SCALE)'s error would be lost: it is not zero and below
-    // 2^-100, or it is beyond 2^126 (or not a number).  Such products belong
-    // into the FP64 accumulator directly.
+    // Products beyond FAR go into the FP64 accumulator: MAX_TERMS of them would
+    // still sum to less than FP32's 2^128.  (In the band above, sums of terms
+    // that each fit would overflow.)
+    static constexpr float FAR = 0x1p120f;
+    static constexpr int MAX_TERMS = 64;
+    // The product a bs's error would be lost: it is not zero and below 2^-100;
+    // or it is beyond FAR (or not a number).  Such products belong into the
+    // FP64 accumulator directly.
     static __device__ __forceinline__ bool far(float a, float bs)
     {
         const float p = fabsf(__fmul_rn(a, bs));
-        return (p < 0x1p-100f && a != 0.0f && bs != 0.0f) || !(p <= 0x1p126f);
+        return (p < 0x1p-100f && a != 0.0f && bs != 0.0f) || !(p <= FAR);
     }
     __device__ __forceinline__ void add(float a, float bs)
     {
@@ -91,8 +102,9 @@ struct Pair {
         hi = s;
         lo = __fadd_rn(lo, __fadd_rn(r, e));
     }
-    __device__ __forceinline__ double value() const { return ((double)hi + (double)lo) * 0x1p-100; }
+    __device__ __forceinline__ double value(double down) const { return ((double)hi + (double)lo) * down; }
 };
+static_assert(RT2D_MAX <= Pair::MAX_TERMS && RT2DP_CHUNK <= Pair::MAX_TERMS, "a pair's terms cannot overflow it");
 
 // Halo and tile rows for an nx x ny grid on `sms` SMs: regions W columns wide,
 // rpw rows per warp and at most maxw warps, halos 4 .. hmax.  The least time
