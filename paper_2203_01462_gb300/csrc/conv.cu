@@ -896,11 +896,15 @@ bool tiled(int W) { return W % 4 == 0 && W * 8 >= (W + 31) / 32 * 32 * 5; }
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
 
-// Whether a block of kernel f can have `bytes` of shared memory on the
-// current device (and its limit raised to them).
-bool smem_ready(const void *f, size_t bytes)
+// Whether a block of kernel f can have `bytes` of shared memory on the current
+// device.  The kernel's limit is raised to `most`, the largest size f is ever
+// launched with, whatever this call's size: the limit belongs to the kernel,
+// and one that followed the calls would let a thread lower it between another
+// thread's call here and its launch.
+bool smem_ready(const void *f, size_t bytes, size_t most)
 {
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess) return true;
+    if (bytes > most) return false;
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) == cudaSuccess) return true;
     cudaGetLastError();
     return false;
 }
@@ -911,7 +915,7 @@ bool fwd_tiled(const float *x, const float *w, const float *bias, float *y, int 
 {
     constexpr int ROWS = TH / WM, BM = 16 * MF * WM, XC = ((ROWS + 2) * 3 * RS / 2 + 11) / 32 * 64 + 40;
     constexpr size_t smem = (2 * 16 * XC + 2 * BM * 152) * sizeof(__nv_bfloat16);
-    if (!smem_ready((const void *)k_conv3_fwd_t<MF, WM>, smem)) return false;
+    if (!smem_ready((const void *)k_conv3_fwd_t<MF, WM>, smem, smem)) return false;
     const dim3 grid((unsigned)((W + 31) / 32 * ((H + ROWS - 1) / ROWS) * B), (co + BM - 1) / BM, splits);
     fdtd::launch_pdl_smem(k_conv3_fwd_t<MF, WM>, grid, 256, smem, st, x, w, bias, y, ci, co, B, H, W, relu, kc, part);
     return true;
@@ -980,12 +984,13 @@ int nn_conv3_dgrad(const float *dy, const float *w, float *dx, int ci, int co, i
     if (!dy || !w || !dx || ci <= 0 || co <= 0 || B <= 0 || H <= 0 || W <= 0) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     const int Kp = (co + 15) / 16 * 16, BM = ci <= 32 ? 32 : 48;
-    // the weights of as many taps at a time as leave room for two blocks per SM
+    // the weights of as many taps at a time as leave room for two blocks per SM; one tap's if none do
+    constexpr size_t two = 113 * 1024, one = 227 * 1024;
     const auto smem = [&](int g) { return (size_t)Kp / 2 * XCD * 4 + (size_t)g * (BM * (Kp + 8) + 8) * 2; };
-    const int G = smem(9) <= 113 * 1024 ? 9 : smem(3) <= 113 * 1024 ? 3 : 1;
+    const int G = smem(9) <= two ? 9 : smem(3) <= two ? 3 : 1;
     const auto f = BM == 32 ? (G == 9 ? k_conv3_dgrad_t<2, 9> : G == 3 ? k_conv3_dgrad_t<2, 3> : k_conv3_dgrad_t<2, 1>)
                             : (G == 9 ? k_conv3_dgrad_t<3, 9> : G == 3 ? k_conv3_dgrad_t<3, 3> : k_conv3_dgrad_t<3, 1>);
-    if (tiled(W) && aligned16(dy) && aligned16(dx) && smem_ready((const void *)f, smem(G))) {
+    if (tiled(W) && aligned16(dy) && aligned16(dx) && smem_ready((const void *)f, smem(G), G == 1 ? one : two)) {
         const dim3 grid((unsigned)((W + 31) / 32 * ((H + TH - 1) / TH) * B), (ci + BM - 1) / BM);
         fdtd::launch_pdl_smem(f, grid, 256, smem(G), st, dy, w, dx, ci, co, Kp, B, H, W, add);
     } else {
