@@ -586,9 +586,7 @@ __global__ void __launch_bounds__(TPB) k_outer_bf16(int M, int N, float alpha, c
 {
     fdtd::pdl_wait();
     fdtd::pdl_trigger();
-    // (64 bits: with N near 2^31 the last block's columns pass the int range)
-    const long long n = (blockIdx.x * (long long)TPB + threadIdx.x) * 4;
-    const int m0 = blockIdx.y * OUTER_M;
+    const int n = (blockIdx.x * TPB + threadIdx.x) * 4, m0 = blockIdx.y * OUTER_M;
     if (n >= N) return;
     auto bf = [](float v) { return __bfloat162float(__float2bfloat16_rn(v)); };
     const float4 b = *reinterpret_cast<const float4 *>(B + n);
