@@ -54,7 +54,8 @@ int nn_col2im3_add(const float *dcol, int C, int B, int H, int W, float *dx, voi
  * (alpha = 1, beta = 0, the same scratch) + nn_bias_act / nn_col2im3_add.
  * nn_conv3_fwd: y = act(w * x + bias), x [ci][B][H][W], w [co][ci 9], y
  * [co][B][H][W].  nn_conv3_dgrad: dx = (add: +=) the input gradient.
- * nn_conv3_wgrad: gw = the weight gradient. */
+ * nn_conv3_wgrad: gw = the weight gradient.  Returns 1 unless 9 ci and
+ * B H W fit an int. */
 int nn_conv3_fwd(const float *x, const float *w, const float *bias, float *y, int ci, int co, int B, int H, int W,
                  int relu, float *work, long long work_elems, void *stream);
 int nn_conv3_dgrad(const float *dy, const float *w, float *dx, int ci, int co, int B, int H, int W, int add, void *stream);

@@ -39,6 +39,7 @@
 // kernels that cost the 8 x 256^2 step 1 % (3.55 -> 3.60 ms).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdint.h>
 
 #include "../../include/surrogate.h"
@@ -894,6 +895,15 @@ inline int slice_blocks(long long n, int per)
 // pixel, and narrower rows would compute more than that in padding.
 bool tiled(int W) { return W % 4 == 0 && W * 8 >= (W + 31) / 32 * 32 * 5; }
 
+// The dimensions of the three products (9 ci, 9 co, B H W) are ints, as
+// nn_gemm_bf16's are; beyond, the choice of the K slices would divide by what
+// is left of them.
+bool sizes_ok(int ci, int co, int B, int H, int W)
+{
+    return ci > 0 && co > 0 && B > 0 && H > 0 && W > 0 && 9LL * ci <= INT_MAX && 9LL * co <= INT_MAX &&
+           (long long)B * H <= INT_MAX && (long long)B * H * W <= INT_MAX;
+}
+
 bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
 
 // Whether a block of kernel f can have `bytes` of shared memory on the current
@@ -959,9 +969,7 @@ int nn_splitk_bf16(int M, long long N, long long K, long long work_elems, long l
 int nn_conv3_fwd(const float *x, const float *w, const float *bias, float *y, int ci, int co, int B, int H, int W,
                  int relu, float *work, long long work_elems, void *stream)
 {
-    if (!x || !w || !bias || !y || ci <= 0 || co <= 0 || B <= 0 || H <= 0 || W <= 0 || work_elems < 0 ||
-        (work_elems > 0 && !work))
-        return 1;
+    if (!x || !w || !bias || !y || !sizes_ok(ci, co, B, H, W) || work_elems < 0 || (work_elems > 0 && !work)) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     const long long P = (long long)B * H * W;
     long long kc = 0;
@@ -981,7 +989,7 @@ int nn_conv3_fwd(const float *x, const float *w, const float *bias, float *y, in
 
 int nn_conv3_dgrad(const float *dy, const float *w, float *dx, int ci, int co, int B, int H, int W, int add, void *stream)
 {
-    if (!dy || !w || !dx || ci <= 0 || co <= 0 || B <= 0 || H <= 0 || W <= 0) return 1;
+    if (!dy || !w || !dx || !sizes_ok(ci, co, B, H, W)) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     const int Kp = (co + 15) / 16 * 16, BM = ci <= 32 ? 32 : 48;
     // the weights of as many taps at a time as leave room for two blocks per SM; one tap's if none do
@@ -1002,8 +1010,7 @@ int nn_conv3_dgrad(const float *dy, const float *w, float *dx, int ci, int co, i
 int nn_conv3_wgrad(const float *dy, const float *x, float *gw, int ci, int co, int B, int H, int W, float *work,
                    long long work_elems, void *stream)
 {
-    if (!dy || !x || !gw || ci <= 0 || co <= 0 || B <= 0 || H <= 0 || W <= 0 || work_elems < 0 || (work_elems > 0 && !work))
-        return 1;
+    if (!dy || !x || !gw || !sizes_ok(ci, co, B, H, W) || work_elems < 0 || (work_elems > 0 && !work)) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     const long long P = (long long)B * H * W;
     long long kc = 0;
