@@ -895,12 +895,12 @@ inline int slice_blocks(long long n, int per)
 // pixel, and narrower rows would compute more than that in padding.
 bool tiled(int W) { return W % 4 == 0 && W * 8 >= (W + 31) / 32 * 32 * 5; }
 
-// The dimensions of the three products (9 ci, 9 co, B H W) are ints, as
+// The dimensions of the three products (9 ci, co, B H W) are ints, as
 // nn_gemm_bf16's are; beyond, the choice of the K slices would divide by what
 // is left of them.
 bool sizes_ok(int ci, int co, int B, int H, int W)
 {
-    return ci > 0 && co > 0 && B > 0 && H > 0 && W > 0 && 9LL * ci <= INT_MAX && 9LL * co <= INT_MAX &&
+    return ci > 0 && co > 0 && B > 0 && H > 0 && W > 0 && 9LL * ci <= INT_MAX &&
            (long long)B * H <= INT_MAX && (long long)B * H * W <= INT_MAX;
 }
 
