@@ -496,15 +496,31 @@ __device__ __forceinline__ void h_tile(const Geo3D &g, const State3D<R> &s, cons
     st4(s.H[2] + q, hz);
 }
 
-// The H half step of the whole grid, bottom up or (zrev) top down; FOLD:
-// with the plane wave's H-face corrections of incident row inc.
+// The tiles of one launch, its planes upwards or downwards.  FP64's smaller
+// tiles can be more rows or planes than a launch has blocks: Part takes them
+// from row y0 and plane z0 on (dz = 1 or -1).  It costs FP32 three registers,
+// and that spills: 2 to 5 % of a step on grids of a wave or two.
+struct Whole {
+    int down;
+    __device__ __forceinline__ int y() const { return blockIdx.y; }
+    __device__ __forceinline__ int z() const { return down ? gridDim.z - 1 - blockIdx.z : blockIdx.z; }
+};
+struct Part {
+    int y0, z0, dz;
+    __device__ __forceinline__ int y() const { return y0 + (int)blockIdx.y; }
+    __device__ __forceinline__ int z() const { return z0 + dz * (int)blockIdx.z; }
+};
+template <typename R>
+using Sweep = std::conditional_t<sizeof(R) == 4, Whole, Part>;
+
+// The H half step; FOLD: with the plane wave's H-face corrections of incident
+// row inc.
 template <typename R, bool FOLD>
 __global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(R) == 4 ? 7 : 24)
-    k_h3d(Geo3D g, State3D<R> s, int slot, Pml3D<R> pm, int zrev, const R *inc)
+    k_h3d(Geo3D g, State3D<R> s, int slot, Pml3D<R> pm, Sweep<R> w, const R *inc)
 {
     wait_previous_grid();
-    const int bz = zrev ? gridDim.z - 1 - blockIdx.z : blockIdx.z;
-    h_tile<Step<R>, R, false, FOLD>(g, s, coef_at<R>(slot), pm, blockIdx.x, blockIdx.y, bz, inc);
+    h_tile<Step<R>, R, false, FOLD>(g, s, coef_at<R>(slot), pm, blockIdx.x, w.y(), w.z(), inc);
 }
 
 // E half step: curl H with backward differences (CPML terms as in the H
@@ -773,11 +789,10 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
 
 template <typename R, int MODE, bool FOLD>
 __global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(R) == 4 ? (MODE == 1 ? 6 : 7) : 24)
-    k_e3d(Geo3D g, State3D<R> s, int slot, Pml3D<R> pm, Step3D<R> a3, int zrev)
+    k_e3d(Geo3D g, State3D<R> s, int slot, Pml3D<R> pm, Step3D<R> a3, Sweep<R> w)
 {
     wait_previous_grid();
-    const int bz = zrev ? gridDim.z - 1 - blockIdx.z : blockIdx.z;
-    e_tile<Step<R>, R, MODE, false, FOLD>(g, s, coef_at<R>(slot), pm, a3, blockIdx.x, blockIdx.y, bz);
+    e_tile<Step<R>, R, MODE, false, FOLD>(g, s, coef_at<R>(slot), pm, a3, blockIdx.x, w.y(), w.z());
 }
 
 // ------------------------------------------------ plane wave (TFSF notes)
@@ -991,23 +1006,33 @@ int launch_step3d(int mode, const Geo3D &g, const State3D<R> &s, int c, const Pm
 {
     using D = Step<R>;
     constexpr int TX = D::BX * D::N;
-    dim3 vblock(D::BX, D::BY, D::BZ),
-        vgrid((g.n[0] + TX - 1) / TX, (g.n[1] + D::BY - 1) / D::BY, (g.n[2] + D::BZ - 1) / D::BZ);
+    const int nx = (g.n[0] + TX - 1) / TX, ny = (g.n[1] + D::BY - 1) / D::BY, nz = (g.n[2] + D::BZ - 1) / D::BZ;
+    const dim3 block(D::BX, D::BY, D::BZ);
     // The H half step sweeps the planes upwards and the E half step
     // downwards (blocks start in blockIdx order), so each launch begins where
     // the previous one ended, on planes whose fields are still in L2.  Each
     // kernel reads only fields it does not write, so the order changes no
     // result.  A forward step of a plane wave adds the face corrections
     // inside the same launches.
-    if (mode == 0 && a.tf_inc) {
-        launch_pdl(k_h3d<R, true>, vgrid, vblock, st, g, s, c, pm, 0, a.tf_inc);
-        launch_pdl(k_e3d<R, 0, true>, vgrid, vblock, st, g, s, c, pm, a, 1);
-    } else {
-        launch_pdl(k_h3d<R, false>, vgrid, vblock, st, g, s, c, pm, 0, (const R *)nullptr);
-        if (mode == 0) launch_pdl(k_e3d<R, 0, false>, vgrid, vblock, st, g, s, c, pm, a, 1);
-        else launch_pdl(k_e3d<R, 1, false>, vgrid, vblock, st, g, s, c, pm, a, 1);
-    }
-    return 2;
+    const bool fold = mode == 0 && a.tf_inc;
+    // rows and planes of tiles of one launch
+    const int MY = sizeof(R) == 4 ? ny : 65535, MZ = sizeof(R) == 4 ? nz : 65535;
+    int launches = 0;
+    for (const bool up : {true, false})
+        for (int z = 0; z < nz; z += MZ)
+            for (int y = 0; y < ny; y += MY) {
+                const dim3 grid(nx, std::min(ny - y, MY), std::min(nz - z, MZ));
+                Sweep<R> w;
+                if constexpr (sizeof(R) == 4) w = Whole{!up};
+                else w = Part{y, up ? z : nz - 1 - z, up ? 1 : -1};
+                if (up && fold) launch_pdl(k_h3d<R, true>, grid, block, st, g, s, c, pm, w, a.tf_inc);
+                else if (up) launch_pdl(k_h3d<R, false>, grid, block, st, g, s, c, pm, w, (const R *)nullptr);
+                else if (fold) launch_pdl(k_e3d<R, 0, true>, grid, block, st, g, s, c, pm, a, w);
+                else if (mode == 0) launch_pdl(k_e3d<R, 0, false>, grid, block, st, g, s, c, pm, a, w);
+                else launch_pdl(k_e3d<R, 1, false>, grid, block, st, g, s, c, pm, a, w);
+                ++launches;
+            }
+    return launches;
 }
 
 
