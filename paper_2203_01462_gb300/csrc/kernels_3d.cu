@@ -38,10 +38,11 @@ namespace {
 // 32 x 8 x 2 nodes (a warp reads 128 contiguous bytes per row).  Shapes
 // (at 768 threads per SM): 8x8x4 at 3 / 8x8x2 at 6 / 4x8x4 at 6 / 8x4x2 at
 // 12 per SM; 8x8x2 and 4x8x4 were fastest, by 3-5 %.  Blocks per SM in FP32
-// (the register budget): H and forward E 7 (72 registers), adjoint E 6 (80).
-// With the CPML terms taken one axis at a time the general path needs about
-// 100 registers unbounded, so these bounds spill (24 B, 128 B in the adjoint
-// E, 40 B in H).  256^3 forward / recompute + adjoint step, us, by blocks of
+// (the register budget): H and forward E 7 (72 registers), adjoint E 6 (80),
+// general instances (see use_plain) H 6.  With the CPML terms taken one axis
+// at a time the general path needs about 100 registers unbounded, so these
+// bounds spill (16 to 24 B, 128 B in the adjoint E, 40 to 48 B in H; general
+// instances 44, 148 and 16 B).  256^3 forward / recompute + adjoint step, us, by blocks of
 // H / E / adjoint E: 6 / 7 / 6 219.1 / 442.5, 7 / 7 / 6 218.4 / 441.1, 8 / 7 / 6
 // 229.0 / 462.8, 6 / 8 / 6 227.7 / 451.4, 6 / 7 / 7 219.1 / 445.9.
 // FP64: one node per thread, blocks of one warp on 8 x 4 nodes.  There the
@@ -347,7 +348,7 @@ __device__ __forceinline__ void cpml_curl(const Geo3D &g, R *const (&psi)[3][2],
 // One tile (bx, by, bz) of the H half step.  COH: loads for the wavefront
 // kernel; FOLD: inc (may then be null) is the plane wave's incident row of
 // this step, whose face corrections are added before the stores.
-template <class SH, typename R, bool COH, bool FOLD>
+template <class SH, typename R, bool COH, bool FOLD, bool PLAIN>
 __device__ __forceinline__ void h_tile(const Geo3D &g, const State3D<R> &s, const Coef<R> &c, const Pml3D<R> &pm,
                                        int bx, int by, int bz, const R *inc)
 {
@@ -357,9 +358,9 @@ __device__ __forceinline__ void h_tile(const Geo3D &g, const State3D<R> &s, cons
     if (i0 >= n0 || j >= n1 || k >= n2) return;
     const long long q = k * g.PP + (long long)j * g.px + i0;
     const long long P = g.px, PP = g.PP;
-    if constexpr (N == 4 && !COH) {
+    if constexpr (PLAIN) {
         // A tile clear of walls, absorbing layer and plane-wave faces (60 % of
-        // them at 256^3): straight code, the same bits.  With its twin in the
+        // them at 256^3): straight code, the same bits (PLAIN: see use_plain).  With its twin in the
         // E half step 225.5 -> 218.4 us per forward step, 453.7 -> 441.1 per
         // recompute + adjoint step; 512 x 512 x 384 1211 -> 1180, 2492 -> 2414.
         // (Instances for tiles with a y- or z-slab only gained nothing more.)
@@ -515,12 +516,12 @@ using Sweep = std::conditional_t<sizeof(R) == 4, Whole, Part>;
 
 // The H half step; FOLD: with the plane wave's H-face corrections of incident
 // row inc.
-template <typename R, bool FOLD>
-__global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(R) == 4 ? 7 : 24)
+template <typename R, bool FOLD, bool PLAIN>
+__global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(R) == 4 ? (PLAIN ? 7 : 6) : 24)
     k_h3d(Geo3D g, State3D<R> s, int slot, Pml3D<R> pm, Sweep<R> w, const R *inc)
 {
     wait_previous_grid();
-    h_tile<Step<R>, R, false, FOLD>(g, s, coef_at<R>(slot), pm, blockIdx.x, w.y(), w.z(), inc);
+    h_tile<Step<R>, R, false, FOLD, PLAIN>(g, s, coef_at<R>(slot), pm, blockIdx.x, w.y(), w.z(), inc);
 }
 
 // E half step: curl H with backward differences (CPML terms as in the H
@@ -529,7 +530,7 @@ __global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(
 // One tile (bx, by, bz) of the E half step.  COH: loads for the wavefront
 // kernel; FOLD (forward): the plane wave's face corrections of row
 // a3.tf_inc (when set) added before the stores.
-template <class SH, typename R, int MODE, bool COH, bool FOLD>
+template <class SH, typename R, int MODE, bool COH, bool FOLD, bool PLAIN>
 __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, const Coef<R> &c, const Pml3D<R> &pm,
                                        const Step3D<R> &a3, int bx, int by, int bz)
 {
@@ -540,11 +541,15 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
     if (i0 >= n0 || j >= n1 || k >= n2) return;
     const long long q = k * g.PP + (long long)j * g.px + i0;
     const long long P = g.px, PP = g.PP;
-    const bool touches = (x0 < g.d0[0] + g.dn[0] && x0 + TX > g.d0[0] && y0 < g.d0[1] + g.dn[1] &&
-                          y0 + TY > g.d0[1] && z0 < g.d0[2] + g.dn[2] && z0 + TZ > g.d0[2]) ||
-                         (MODE == 0 && x0 < g.s1[0] && x0 + TX > g.s0[0] && y0 < g.s1[1] && y0 + TY > g.s0[1] &&
-                          z0 < g.s1[2] && z0 + TZ > g.s0[2]);
-    if constexpr (N == 4 && !COH) {
+    auto touch = [&]() {  // the tile has nodes of the design box or the source
+        return (x0 < g.d0[0] + g.dn[0] && x0 + TX > g.d0[0] && y0 < g.d0[1] + g.dn[1] && y0 + TY > g.d0[1] &&
+                z0 < g.d0[2] + g.dn[2] && z0 + TZ > g.d0[2]) ||
+               (MODE == 0 && x0 < g.s1[0] && x0 + TX > g.s0[0] && y0 < g.s1[1] && y0 + TY > g.s0[1] &&
+                z0 < g.s1[2] && z0 + TZ > g.s0[2]);
+    };
+    bool touches = false;  // (asked early only where it decides: across the loads it costs registers)
+    if constexpr (PLAIN) touches = touch();
+    if constexpr (PLAIN) {
         // a tile clear of walls, absorbing layer, design box, source and plane-wave faces
         const int np1 = g.npml + 1;
         bool plain = !touches && x0 >= np1 && x0 + TX <= n0 - np1 && y0 >= np1 && y0 + TY <= n1 - np1 && z0 >= np1 &&
@@ -647,6 +652,7 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
         if (cc == 1) return j <= n1 - 2 && imid && kmid;
         return k <= n2 - 2 && imid && jmid;
     };
+    if constexpr (!PLAIN) touches = touch();
     // (FP64 reciprocals, some fifteen operations, come from the host; FP32's
     // are rounded from FP32 operands)
     constexpr bool F64 = sizeof(R) == 8;
@@ -787,12 +793,12 @@ __device__ __forceinline__ void e_tile(const Geo3D &g, const State3D<R> &s, cons
     }
 }
 
-template <typename R, int MODE, bool FOLD>
+template <typename R, int MODE, bool FOLD, bool PLAIN>
 __global__ void __launch_bounds__(Step<R>::BX *Step<R>::BY *Step<R>::BZ, sizeof(R) == 4 ? (MODE == 1 ? 6 : 7) : 24)
     k_e3d(Geo3D g, State3D<R> s, int slot, Pml3D<R> pm, Step3D<R> a3, Sweep<R> w)
 {
     wait_previous_grid();
-    e_tile<Step<R>, R, MODE, false, FOLD>(g, s, coef_at<R>(slot), pm, a3, blockIdx.x, w.y(), w.z());
+    e_tile<Step<R>, R, MODE, false, FOLD, PLAIN>(g, s, coef_at<R>(slot), pm, a3, blockIdx.x, w.y(), w.z());
 }
 
 // ------------------------------------------------ plane wave (TFSF notes)
@@ -947,7 +953,7 @@ __global__ void __launch_bounds__(TBX *TBY *TBZ, sizeof(R) == 4 ? WAVE_MINB : 1)
         if (!isE) {
             const R *inc = (MODE == 0 && w.tf) ? w.tf + (long long)(w.n0 + t) * w.tf_row : nullptr;
 #pragma unroll 1
-            for (int bx = bx0; bx < bx1; ++bx) h_tile<Tile4, R, true, true>(g, s, c, pm, bx, by, sl, inc);
+            for (int bx = bx0; bx < bx1; ++bx) h_tile<Tile4, R, true, true, false>(g, s, c, pm, bx, by, sl, inc);
         } else {
             Step3D<R> a = a0;
             if (MODE == 0) {
@@ -962,7 +968,7 @@ __global__ void __launch_bounds__(TBX *TBY *TBZ, sizeof(R) == 4 ? WAVE_MINB : 1)
                 a.rec = w.rec + (long long)(m - 1 - w.rec0) * 3 * g.Mdi;
             }
 #pragma unroll 1
-            for (int bx = bx0; bx < bx1; ++bx) e_tile<Tile4, R, MODE, true, true>(g, s, c, pm, a, bx, by, sl);
+            for (int bx = bx0; bx < bx1; ++bx) e_tile<Tile4, R, MODE, true, true, false>(g, s, c, pm, a, bx, by, sl);
         }
         __syncthreads();
         // E items of the last step have no reader in this launch
@@ -1000,9 +1006,10 @@ template void launch_tfsf_column<float>(const Geo3D &, const Pml3D<float> &, flo
 template void launch_tfsf_column<double>(const Geo3D &, const Pml3D<double> &, double, double, double,
                                          const double *, int, double *, double *, cudaStream_t);
 
-template <typename R>
-int launch_step3d(int mode, const Geo3D &g, const State3D<R> &s, int c, const Pml3D<R> &pm,
-                  const Step3D<R> &a, cudaStream_t st)
+// The launches of one step; PLAIN as in h_tile.
+template <typename R, bool PLAIN>
+int sweep_step3d(int mode, const Geo3D &g, const State3D<R> &s, int c, const Pml3D<R> &pm, const Step3D<R> &a,
+                 cudaStream_t st)
 {
     using D = Step<R>;
     constexpr int TX = D::BX * D::N;
@@ -1025,14 +1032,51 @@ int launch_step3d(int mode, const Geo3D &g, const State3D<R> &s, int c, const Pm
                 Sweep<R> w;
                 if constexpr (sizeof(R) == 4) w = Whole{!up};
                 else w = Part{y, up ? z : nz - 1 - z, up ? 1 : -1};
-                if (up && fold) launch_pdl(k_h3d<R, true>, grid, block, st, g, s, c, pm, w, a.tf_inc);
-                else if (up) launch_pdl(k_h3d<R, false>, grid, block, st, g, s, c, pm, w, (const R *)nullptr);
-                else if (fold) launch_pdl(k_e3d<R, 0, true>, grid, block, st, g, s, c, pm, a, w);
-                else if (mode == 0) launch_pdl(k_e3d<R, 0, false>, grid, block, st, g, s, c, pm, a, w);
-                else launch_pdl(k_e3d<R, 1, false>, grid, block, st, g, s, c, pm, a, w);
+                if (up && fold) launch_pdl(k_h3d<R, true, PLAIN>, grid, block, st, g, s, c, pm, w, a.tf_inc);
+                else if (up) launch_pdl(k_h3d<R, false, PLAIN>, grid, block, st, g, s, c, pm, w, (const R *)nullptr);
+                else if (fold) launch_pdl(k_e3d<R, 0, true, PLAIN>, grid, block, st, g, s, c, pm, a, w);
+                else if (mode == 0) launch_pdl(k_e3d<R, 0, false, PLAIN>, grid, block, st, g, s, c, pm, a, w);
+                else launch_pdl(k_e3d<R, 1, false, PLAIN>, grid, block, st, g, s, c, pm, a, w);
                 ++launches;
             }
     return launches;
+}
+
+// Whether a step runs the PLAIN instances (see h_tile).  In tiles that are not
+// plain they are the slower ones (their test; H at 72 registers spills), and
+// on a few waves such tiles decide.  Forward / adjoint step in us, general and
+// plain: 40 x 85 x 104 16.2 / 34.9 and 17.0 / 36.7, 70 x 90 x 81 (plane wave) 19.2 /
+// 40.4 and 20.1 / 42.4, 63 x 171 x 141 26.2 / 54.1 and 26.3 / 55.0, 128^3 29.5 /
+// 61.5 and 28.9 / 61.4, 180^3 87.6 / 178.6 and 84.6 / 172.9, 256^3 221.7 / 460.5
+// and 215.7 / 448.6.  From 2^21 nodes on plain is faster, whatever the share of
+// plain tiles (60 x 100 x 600, none: 67.8 / 140.0 and 66.8 / 139.2), below where
+// a fifth of the tiles is (234 x 76 x 38 14.0 / 28.7 and 13.7 / 28.7; 136 x 81 x 64,
+// 17 %: 17.8 / 38.5 and 18.3 / 39.4).  With a plane wave's faces, whose tiles
+// are not plain either, the line lies higher: forward 128^3 30.1 and 30.1, 99 x
+// 202 x 150 (3.0e6 nodes) 66.4 and 66.6, 132 x 236 x 120 (3.7e6) 67.3 and 65.8.
+bool use_plain(const Geo3D &g, bool fold)
+{
+    const long long nodes = (long long)g.n[0] * g.n[1] * g.n[2];
+    if (fold) return nodes >= 7LL << 19;
+    if (nodes >= 1LL << 21) return true;
+    const int side[3] = {TX, TBY, TBZ}, np1 = g.npml + 1;
+    long long tiles = 1, plain = 1;
+    for (int a = 0; a < 3; ++a) {
+        const int first = (np1 + side[a] - 1) / side[a], last = (g.n[a] - np1) / side[a];  // tiles clear of the layer
+        tiles *= (g.n[a] + side[a] - 1) / side[a];
+        plain *= std::max(0, last - first);
+    }
+    return 5 * plain >= tiles;
+}
+
+template <typename R>
+int launch_step3d(int mode, const Geo3D &g, const State3D<R> &s, int c, const Pml3D<R> &pm,
+                  const Step3D<R> &a, cudaStream_t st)
+{
+    if constexpr (sizeof(R) == 4) {
+        if (use_plain(g, mode == 0 && a.tf_inc)) return sweep_step3d<R, true>(mode, g, s, c, pm, a, st);
+    }
+    return sweep_step3d<R, false>(mode, g, s, c, pm, a, st);
 }
 
 
