@@ -252,10 +252,12 @@ fdtd_status fdtd_set_filter_width(fdtd_ctx *ctx, double sigma);
 
 /* Time steps per launch.  In-plane 2D contexts (pol = FDTD_POL_INPLANE):
  * left unset, up to 8 steps per launch (4 in FP64) by temporal blocking, as
- * for E_z below (the paper's 291^2 and 491^2 geometries: 4.9 and 5.9 us per
- * forward step with one launch per half step, 1.4 and 2.3 blocked; the
- * adjoint's sensitivities are summed by a second kernel from the records of
- * up to 32 steps).  1: one launch per half step.  With more than one, a run
+ * for E_z below, in FP32 and on FP64 grids that are small or largely design
+ * box, and one launch per half step on the others (FP32, the paper's 291^2 and
+ * 491^2 geometries: 4.9 and 5.9 us per forward step with one launch per half
+ * step, 1.4 and 2.3 blocked; FP64, 2000^2 with a 592^2 design box: 152 and 203;
+ * the blocked adjoint's sensitivities are summed by a second kernel from the
+ * records of up to 32 steps).  1: one launch per half step.  With more than one, a run
  * of steps is one cooperative launch, one block per SM, whose half steps are
  * separated by grid-wide barriers with bounded waits (FDTD_ETIMEOUT from
  * fdtd_sync if one gives up), about 12 us per 491^2 step; such passes are not

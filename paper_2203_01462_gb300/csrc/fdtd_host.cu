@@ -1061,11 +1061,32 @@ struct CtxP final : fdtd_ctx {
     char *F_base[2] = {nullptr, nullptr}, *A_base[2] = {nullptr, nullptr};
     int curF = 0, curA = 0;
     // Temporal blocking (kernels_rt2dp.cu), the default (steps per launch not
-    // set) where it was measured faster.
-    bool rt_ok = false;
+    // set) where rt_auto says so.
+    bool rt_ok = false, rt_auto = false;
     int rt_sms = 0;
     R *rt_coef[2] = {nullptr, nullptr};
     bool rt() const { return rt_ok && multi_steps == 0; }
+    // In FP32 blocked launches were faster on every grid measured (34^2 to
+    // 3000^2, thin ones too).  In FP64 the FP64 units bound both forms: the
+    // blocked one advances halo rows and columns twice but reads the Drude
+    // coefficients, which the other works out anew on every design edge and
+    // step.  So it wins where the tiles are one wave, and otherwise where the
+    // design box is enough of the grid.  Forward / adjoint step with
+    // checkpoints in us, one launch per half step and blocked, by the box's
+    // share of the nodes: 400^2 2 % 9.9 / 20.7 and 11.2 / 24.6, 18 % 13.1 / 30.6
+    // and 12.7 / 29.2; 491^2 8 % 15.1 / 33.6 and 17.2 / 36.6, 32 % 20.6 / 47.9 and
+    // 18.9 / 38.5; 1000^2 9 % 43.6 / 94.7 and 53.6 / 109.6, 77 % 98 / 249 and 84 /
+    // 191; 2000^2 9 % 152 / 320 and 203 / 414, 79 % 366 / 933 and 319 / 735.  The
+    // line follows 90 random shapes; on the wrong side of it are a few, by up to
+    // 9 % (371 x 166 with 15 %, 586 x 93 with 29 %).
+    bool blocks_by_default() const
+    {
+        if (sizeof(R) == 4) return true;
+        const Rt2DPlan p = rt2dp_plan<R>(cfg.nx, cfg.ny, 152);
+        if (p.bx * p.by <= 152) return true;
+        const double nodes = (double)cfg.nx * cfg.ny, box = (double)box_count(cfg.design_lo, cfg.design_hi, 2);
+        return box >= std::min(0.35, 0.1 + nodes / 5e6) * nodes;
+    }
     Rt2DPlan rt_plan() const { return rt2dp_plan<R>(geo.nx, geo.ny, rt_sms); }
     // Adjoint records of a chunk of steps, and the adjoint J and E before it.
     R *arec = nullptr, *jsens[2] = {nullptr, nullptr}, *eprev[2] = {nullptr, nullptr};
@@ -1186,16 +1207,19 @@ struct CtxP final : fdtd_ctx {
             geo.s1[a] = c.src_hi[a];
         }
         const long long N = c.nsteps;
-        for (int b = 0; b < 2; ++b) carve_state(cv, F[b], F_base[b]);
-        for (int b = 0; b < 2; ++b) carve_state(cv, A[b], A_base[b]);
+        rt_auto = blocks_by_default();
+        for (int b = 0; b < 1 + rt_auto; ++b) carve_state(cv, F[b], F_base[b]);
+        for (int b = 0; b < 1 + rt_auto; ++b) carve_state(cv, A[b], A_base[b]);
         rho = cv.take<R>(Md);
         rho_t[0] = cv.take<R>((size_t)geo.Mdi[0]);
         rho_t[1] = cv.take<R>((size_t)geo.Mdi[1]);
-        for (int cc = 0; cc < 2; ++cc) rt_coef[cc] = cv.take<R>(5 * (size_t)geo.Mdi[cc]);
-        arec = cv.take<R>((size_t)RT2DP_CHUNK * Mdi_all());
-        for (int cc = 0; cc < 2; ++cc) {
-            jsens[cc] = cv.take<R>((size_t)geo.Mdi[cc]);
-            eprev[cc] = cv.take<R>((size_t)geo.Mdi[cc]);
+        if (rt_auto) {
+            for (int cc = 0; cc < 2; ++cc) rt_coef[cc] = cv.take<R>(5 * (size_t)geo.Mdi[cc]);
+            arec = cv.take<R>((size_t)RT2DP_CHUNK * Mdi_all());
+            for (int cc = 0; cc < 2; ++cc) {
+                jsens[cc] = cv.take<R>((size_t)geo.Mdi[cc]);
+                eprev[cc] = cv.take<R>((size_t)geo.Mdi[cc]);
+            }
         }
         rstage = cv.take<R>(Md);
         G[0] = cv.take<double>((size_t)geo.Mdi[0]);
@@ -1239,7 +1263,7 @@ struct CtxP final : fdtd_ctx {
         launch_zero_bytes(err, 4 * sizeof(unsigned), st);
         ++launches;
         multi_fits = stepp_multi_fits<R>(geo);
-        rt_ok = rt2dp_ready<R>();
+        rt_ok = rt_auto && rt2dp_ready<R>();
         {
             int dev = 0;
             cudaGetDevice(&dev);
