@@ -1207,6 +1207,7 @@ struct CtxP final : fdtd_ctx {
             geo.s1[a] = c.src_hi[a];
         }
         const long long N = c.nsteps;
+        const long long K = c.snapshot_every, nrec = K > 0 ? std::min<long long>(K, N) : N;  // steps recorded at a time
         rt_auto = blocks_by_default();
         for (int b = 0; b < 1 + rt_auto; ++b) carve_state(cv, F[b], F_base[b]);
         for (int b = 0; b < 1 + rt_auto; ++b) carve_state(cv, A[b], A_base[b]);
@@ -1215,7 +1216,7 @@ struct CtxP final : fdtd_ctx {
         rho_t[1] = cv.take<R>((size_t)geo.Mdi[1]);
         if (rt_auto) {
             for (int cc = 0; cc < 2; ++cc) rt_coef[cc] = cv.take<R>(5 * (size_t)geo.Mdi[cc]);
-            arec = cv.take<R>((size_t)RT2DP_CHUNK * Mdi_all());
+            arec = cv.take<R>((size_t)std::min<long long>(RT2DP_CHUNK, nrec) * Mdi_all());
             for (int cc = 0; cc < 2; ++cc) {
                 jsens[cc] = cv.take<R>((size_t)geo.Mdi[cc]);
                 eprev[cc] = cv.take<R>((size_t)geo.Mdi[cc]);
@@ -1226,8 +1227,7 @@ struct CtxP final : fdtd_ctx {
         G[1] = cv.take<double>((size_t)geo.Mdi[1]);
         gstage = cv.take<double>(Md);
         gap_hist = cv.take<R>((size_t)(N + 1) * (Mg ? Mg : 1));
-        const long long K = c.snapshot_every;
-        rec = cv.take<R>((size_t)(K > 0 ? std::min<long long>(K, N) : N) * Mdi_all());
+        rec = cv.take<R>((size_t)nrec * Mdi_all());
         nsnap = K > 0 ? (int)((N + K - 1) / K) : 0;
         snap_stride = snapshot_bytes<R>(c.snapshot_dtype, state_bytes);
         snaps = cv.take<char>((size_t)nsnap * snap_stride);
