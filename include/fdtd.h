@@ -72,7 +72,8 @@ typedef enum fdtd_status {
  * (lossy: the recomputed forward fields, hence the gradient, carry the
  * rounding of the restart). */
 enum { FDTD_SNAP_F32 = 0, FDTD_SNAP_BF16 = 1, FDTD_SNAP_F16 = 2 };
-/* Sensitivity accumulator: FDTD_ACC_F64 (one FP64 sum per design node).
+/* Sensitivity accumulator: FDTD_ACC_F64 (one FP64 sum per design node; see
+ * fdtd_set_steps_per_launch for what 2D FP32 runs add to it at a time).
  * FDTD_ACC_COMP_F32 (a compensated FP32 pair) is reserved and rejected with
  * FDTD_EINVAL: it would move the same 16 bytes per node and step. */
 enum { FDTD_ACC_F64 = 0, FDTD_ACC_COMP_F32 = 1 };
@@ -257,8 +258,8 @@ fdtd_status fdtd_set_filter_width(fdtd_ctx *ctx, double sigma);
  * 491^2 geometries: 4.9 and 5.9 us per forward step with one launch per half
  * step, 1.4 and 2.3 blocked; FP64, 2000^2 with a 592^2 design box: 152 and 203;
  * the blocked adjoint's sensitivities are summed by a second kernel from the
- * records of up to 32 steps).  1: one launch per half step.  With more than one, a run
- * of steps is one cooperative launch, one block per SM, whose half steps are
+ * records of up to 32 steps).  1: one launch per half step.  With more than
+ * one, a run of steps is one cooperative launch, one block per SM, whose half steps are
  * separated by grid-wide barriers with bounded waits (FDTD_ETIMEOUT from
  * fdtd_sync if one gives up), about 12 us per 491^2 step; such passes are not
  * replayed as CUDA graphs.  W~ and the gap history are bit-identical in all
@@ -277,8 +278,10 @@ fdtd_status fdtd_set_filter_width(fdtd_ctx *ctx, double sigma);
  * the gap history (for a Courant number that is a power of two; to rounding
  * otherwise), except on FP32 grids of at most one 32 x 32 tile per SM
  * and with steps > 1, where a Drude node's two products are rounded in the
- * other order; the gradient's FP32 sums of one launch are kept as exact
- * pairs before they go into the FP64 accumulator (1e-14 relative).
+ * other order.  The FP32 gradient's products of one launch (in plane: of up to
+ * 32 steps) are added up in FP32 words that keep the rounding errors before
+ * they go into the FP64 accumulators: about as far from the exact sums as FP64
+ * additions would be (1e-15 relative, rms).
  *
  * 3D contexts ignore the setting (see fdtd_set_wavefront). */
 fdtd_status fdtd_set_steps_per_launch(fdtd_ctx *ctx, int steps);

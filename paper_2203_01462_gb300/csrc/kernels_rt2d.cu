@@ -53,7 +53,7 @@ struct Shape {
     static constexpr int VX = sizeof(R) == 4 ? 2 : 1;
     static constexpr int RPW = sizeof(R) == 4 ? 2 : 1;
     static constexpr int W = 32 * VX;   // region width
-    static constexpr int MAXW = sizeof(R) == 4 ? 16 : 24;  // warps per block (FP32: 128 registers a thread, no spills)
+    static constexpr int MAXW = sizeof(R) == 4 ? 16 : 24;  // warps per block (FP32: 128 registers a thread)
 };
 
 // Shared memory of one block (in words of R unless noted), in this order:
@@ -79,7 +79,14 @@ constexpr int GAP_STAGED = 256;
 // change with the kernel that computes them.
 // NB: blocks per SM the registers have to leave room for; 0: one, and only
 // the general kind of region (see launch_rt2d).
-template <typename R, int MODE, int FORM, int NB>
+// FULL (FP32 adjoint): a launch's sums go into the FP64 accumulator with all
+// they hold, or rounded to 2^-49, which saves one of three conversions to FP64
+// per node and launch.  Against the exact sums (rt_common.cuh; ten grids, rms)
+// the rounded ones are as far off as FP64 sums are, 0.6 to 1.1 times, with up
+// to 6 steps a launch, and 0.7 to 1.15 times with 8: there FULL is 0.4 to 0.65
+// times.  us per evaluation, not FULL / FULL: 316^2 (8 steps) 9106 / 9207, 530 x 303
+// (4 steps) 4910 / 5077.
+template <typename R, int MODE, int FORM, int NB, bool FULL>
 __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
     k_rt2d(const __grid_constant__ Geo2D g, const __grid_constant__ State2D<R> in,
            const __grid_constant__ State2D<R> out, int slot, const __grid_constant__ Pml1D<R> px,
@@ -201,7 +208,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
 #pragma unroll
         for (int v = 0; v < VX; ++v) {
             G[r][v] = 0.0;
-            gp[r][v] = Pair{0.0f, 0.0f};
+            gp[r][v] = Pair{};
         }
         if (PL || ((unsigned)j < (unsigned)ny && cin)) {
             const long long q = (long long)j * P + i0;
@@ -319,7 +326,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
     const bool k1 = w.kappa1 != 0;
     R *rec = nullptr;
     if (MODE == 0 && w.rec) rec = w.rec + (long long)(w.n0 - w.rec0) * w.Mdi;
-    const R *srp = srec + (size_t)tid * VX;  // this thread's record of row 0, step 0
+    R *srp = srec + (size_t)tid * VX;  // this thread's record of row 0, step 0
 
     // The step loop, one instance per kind of block (XP / YP: its region
     // meets the columns' / rows' absorbing layer, DR: the design box), so
@@ -521,7 +528,13 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
 #pragma unroll
                     for (int r = 0; r < RPW; ++r)
 #pragma unroll
-                        for (int v = 0; v < VX; ++v) gp[r][v].add(em[r][v], term[r][v] * w.ps.up);
+                        for (int v = 0; v < VX; ++v) {
+                            // (two blocks per SM: no registers for the products'
+                            // errors, which take the place of the step's record)
+                            if constexpr (NB == 2)
+                                srp[(size_t)(t * RPW + r) * nth * VX + v] = gp[r][v].add_rounded(em[r][v], term[r][v] * w.ps.up);
+                            else gp[r][v].add(em[r][v], term[r][v] * w.ps.up);
+                        }
                 }
             }
 #pragma unroll
@@ -565,6 +578,14 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
         else run(No{}, No{}, No{});
     }
 
+    if constexpr (MODE == 1 && NB == 2 && !V) {
+        if (ownw && (D || dru))
+            for (int t = 0; t < T; ++t)
+#pragma unroll
+                for (int r = 0; r < RPW; ++r)
+#pragma unroll
+                    for (int v = 0; v < VX; ++v) gp[r][v].c += srp[(size_t)(t * RPW + r) * nth * VX + v];
+    }
     // ---- store the tile's own nodes into the other buffer of the pair
 #pragma unroll
     for (int r = 0; r < RPW; ++r) {
@@ -581,7 +602,7 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, NB > 0 ? NB : 1)
                 for (int v = 0; v < VX; ++v) {
                     if (!(sens >> (r * VX + v) & 1u)) continue;
                     if constexpr (F64) w.G[d[r] + v] = G[r][v];
-                    else w.G[d[r] + v] += gp[r][v].value(w.ps.down);
+                    else w.G[d[r] + v] += FULL ? gp[r][v].value(w.ps.down) : gp[r][v].value49(w.ps.down);
                 }
             }
         }
@@ -672,12 +693,26 @@ Rt2DPlan rt2d_plan(int nx, int ny, int sms, int steps)
 }
 
 template <typename R, int NB>
+using Kernel = decltype(&k_rt2d<R, 0, 0, NB, false>);
+
+// The instance for a mode, a rounding form and a halo.
+template <typename R, int NB>
+Kernel<R, NB> instance(int mode, int form, int halo)
+{
+    if (mode == 0) return form ? k_rt2d<R, 0, 1, NB, false> : k_rt2d<R, 0, 0, NB, false>;
+    if constexpr (sizeof(R) == 4)
+        if (halo > 6) return form ? k_rt2d<R, 1, 1, NB, true> : k_rt2d<R, 1, 0, NB, true>;
+    return form ? k_rt2d<R, 1, 1, NB, false> : k_rt2d<R, 1, 0, NB, false>;
+}
+
+template <typename R, int NB>
 bool allow(size_t b)
 {
-    return cudaFuncSetAttribute(k_rt2d<R, 0, 0, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) == cudaSuccess &&
-           cudaFuncSetAttribute(k_rt2d<R, 1, 0, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) == cudaSuccess &&
-           cudaFuncSetAttribute(k_rt2d<R, 0, 1, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) == cudaSuccess &&
-           cudaFuncSetAttribute(k_rt2d<R, 1, 1, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) == cudaSuccess;
+    bool ok = true;
+    for (int q = 0; q < 8; ++q)
+        ok = ok && cudaFuncSetAttribute(instance<R, NB>(q & 1, q >> 1 & 1, q & 4 ? RT2D_MAX : 4),
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) == cudaSuccess;
+    return ok;
 }
 
 template <typename R>
@@ -701,9 +736,7 @@ void launch_nb(int mode, const Geo2D &g, const State2D<R> &in, const State2D<R> 
     const int Mg = g.gnx * g.gny;
     const size_t smem = smem_words<R>(p.nw, w.count, mode == 1 && Mg <= GAP_STAGED ? Mg : 0, mode) * sizeof(R);
     const dim3 block(32, p.nw), grid(p.bx, p.by);
-    const auto k = mode == 0 ? (p.form ? k_rt2d<R, 0, 1, NB> : k_rt2d<R, 0, 0, NB>)
-                             : (p.form ? k_rt2d<R, 1, 1, NB> : k_rt2d<R, 1, 0, NB>);
-    launch_pdl_smem(k, grid, block, smem, st, g, in, out, slot, px, py, w);
+    launch_pdl_smem(instance<R, NB>(mode, p.form, p.halo), grid, block, smem, st, g, in, out, slot, px, py, w);
 }
 
 // Tiles whose region is plain background (V; those of the source's rows counted too).

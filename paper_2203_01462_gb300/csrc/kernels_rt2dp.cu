@@ -461,11 +461,11 @@ __global__ void __launch_bounds__(128) k_rt2dp_sens(int slot, long long M0, long
     ld16(ep, eo);
     ld16(jp, jo);
     double g[V];
-    Pair gp[V];
+    PairSum gp[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         g[v] = 0.0;
-        gp[v] = Pair{0.0f, 0.0f};
+        gp[v] = PairSum{};
     }
     for (int t0 = 0; t0 < count; t0 += U) {
         R en[U][V], em[U][V];
@@ -505,10 +505,17 @@ __global__ void __launch_bounds__(128) k_rt2dp_sens(int slot, long long M0, long
                             en[k][v] = 0.0f;
                         }
             }
+            // (steps past the last add zero)
 #pragma unroll
-            for (int k = 0; k < U; ++k)
+            for (int v = 0; v < V; ++v) {
+                Pair q{};
 #pragma unroll
-                for (int v = 0; v < V; ++v) gp[v].add(em[k][v], en[k][v] * ps.up);
+                for (int k = 0; k < U; ++k) {
+                    q.add(em[k][v], en[k][v] * ps.up);
+                    if (k % 4 == 3) gp[v].errors(q);
+                }
+                gp[v].merge(q);
+            }
         }
     }
     if (!inside) return;
