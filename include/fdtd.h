@@ -271,8 +271,9 @@ fdtd_status fdtd_set_filter_width(fdtd_ctx *ctx, double sigma);
  * in FP32 as suits the grid) by temporal blocking: a block holds a tile of
  * the grid and a halo of that many nodes in registers, advances all the
  * steps there and writes back its tile, so no block waits for another.  Left
- * unset, FP32 grids and FP64 grids of at most 2^20 nodes run so and larger
- * FP64 ones with one launch per step (316^2 FP32: 6.9 us per forward step with one launch
+ * unset, FP32 grids and FP64 grids of at most 2^20 nodes (beyond 450 000, with
+ * a design box of 4 % of them) run so and the other FP64 ones with one launch
+ * per step (316^2 FP32: 6.9 us per forward step with one launch
  * per step, 1.0 blocked; 160^2 FP64: 12.1 and 3.3).  Results of a run left
  * unset are those of one launch per step bit for bit in the fields, W~ and
  * the gap history (for a Courant number that is a power of two; to rounding

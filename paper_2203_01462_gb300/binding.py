@@ -298,9 +298,8 @@ class Solver:
 
     def set_steps_per_launch(self, steps: int) -> None:
         """Time steps per launch.  Left unset: temporal blocking on tiles with a
-        halo held in registers (up to 8 steps, 4 in FP64) on E_z grids in FP32 or
-        of at most 2^20 nodes, and in-plane grids in FP32, small, or largely
-        design box; one launch per step (in-plane: per half step) on the
+        halo held in registers (up to 8 steps, 4 in FP64) on grids in FP32, and in
+        FP64 on small ones and those with enough design box (fdtd.h); one launch per step (in-plane: per half step) on the
         others.  1: one launch per step everywhere.  More: E_z, blocked with at
         most that many steps; in-plane, a cooperative launch with grid barriers."""
         _check(self.lib.fdtd_set_steps_per_launch(self.ctx, int(steps)), "fdtd_set_steps_per_launch")

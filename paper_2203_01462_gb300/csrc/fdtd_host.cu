@@ -678,8 +678,15 @@ struct Ctx2D final : fdtd_ctx {
             // 23.2 / 25 against 13.2 / 19.6 (21.2 forward with the L2 window,
             // which the blocked launches do not take), 4096^2 77 / 86 against
             // 47 / 69; FP64 160^2 12.1 / 15.1 against 3.3 / 3.3, 1000^2 52 /
-            // 72 against 49 / 53.
-            rt_auto = sizeof(R) == 4 || ncells <= 1LL << 20;
+            // 72 against 49 / 53.  In FP64 the halo's nodes cost what the Drude
+            // coefficients, worked out anew by each step otherwise, save: with
+            // checkpoints and a design box of 0.1 / 4 / 8 % of the nodes, forward
+            // / adjoint, 600^2 19.2 / 36.9 against 18.1 / 36.4 with 0.1 %, 700^2
+            // 22.0 / 46.0 against 23.5 / 47.1, 1000^2 39.7 / 76.4 against 41.9 /
+            // 84.4 with 0.1 and 45.1 / 88.6 against 42.8 / 87.6 with 4 %, 1020^2
+            // 44.3 / 89.0 against 45.0 / 91.9 with 4 and 47.0 / 100.6 against 46.1
+            // / 95.4 with 8 %.
+            rt_auto = sizeof(R) == 4 || (ncells <= 1LL << 20 && (ncells <= 450000 || 25 * Md >= ncells));
         }
         return cuda_ok(cudaStreamSynchronize(st));
     }
