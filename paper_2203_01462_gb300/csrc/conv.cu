@@ -36,7 +36,10 @@
 // step 0.98 -> 0.80 ms, 256^2 prediction 0.34 -> 0.25.  The short kernels and
 // the weight gradient, which leaves room on the SMs, also let their
 // successor's blocks in while they run; for the forward and input-gradient
-// kernels that cost the 8 x 256^2 step 1 % (3.55 -> 3.60 ms).
+// kernels that cost the 8 x 256^2 step 1 % (3.55 -> 3.60 ms), and for the GEMMs
+// and the passes around them (nn.cu) up to a third of the FP32 network: 8 x
+// 256^2 training step 31.6 ms with, 28.5 without, 2 x 96^2 at base 64 6.10 and
+// 4.65, 512^2 at base 8 6.37 and 4.68 (29.4, 5.20 and 5.31 as plain launches).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <limits.h>

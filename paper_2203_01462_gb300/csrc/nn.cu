@@ -41,7 +41,6 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, float alpha, 
                                               int kc, float *part)
 {
     fdtd::pdl_wait();
-    fdtd::pdl_trigger();
     __shared__ float As[GK][GT + 4];
     __shared__ float Bs[GK][GT + 4];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -103,7 +102,6 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, float alpha, 
 __global__ void k_splitk_sum(float *C, int ldc, const float *__restrict__ part, int M, int N, int S, float beta)
 {
     fdtd::pdl_wait();
-    fdtd::pdl_trigger();
     const long long n = (long long)M * N;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         float acc = part[e];
@@ -119,7 +117,6 @@ __global__ void k_splitk_sum(float *C, int ldc, const float *__restrict__ part, 
 __global__ void k_im2col3(const float *x, int C, int B, int H, int W, float *col)
 {
     fdtd::pdl_wait();
-    fdtd::pdl_trigger();
     const int HW = H * W;
     const long long P = (long long)B * HW, n = (long long)C * P;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -142,7 +139,6 @@ __global__ void k_im2col3(const float *x, int C, int B, int H, int W, float *col
 __global__ void k_col2im3(const float *col, int C, int B, int H, int W, float *dx)
 {
     fdtd::pdl_wait();
-    fdtd::pdl_trigger();
     const long long P = (long long)B * H * W, n = (long long)C * P;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(e / P);
@@ -163,7 +159,6 @@ __global__ void k_col2im3(const float *col, int C, int B, int H, int W, float *d
 __global__ void k_bias_act(float *y, const float *bias, int Cout, long long P, int relu)
 {
     fdtd::pdl_wait();
-    fdtd::pdl_trigger();
     const long long n = (long long)Cout * P;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         float v = y[e] + bias[e / P];
@@ -501,7 +496,6 @@ __global__ void __launch_bounds__(256) k_gemm_bf16(int M, int N, int K, float al
                                                    float *C, int ldc, int kc, float *part)
 {
     fdtd::pdl_wait();
-    fdtd::pdl_trigger();
     __shared__ __align__(16) __nv_bfloat16 As[BM][BKP];
     __shared__ __align__(16) __nv_bfloat16 Bs[BN][BKP];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
