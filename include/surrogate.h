@@ -62,6 +62,18 @@ int nn_conv3_dgrad(const float *dy, const float *w, float *dx, int ci, int co, i
 int nn_conv3_wgrad(const float *dy, const float *x, float *gw, int ci, int co, int B, int H, int W, float *work,
                    long long work_elems, void *stream);
 
+/* The same with scratch for the im2col matrix, 9 ci B H W words: where the
+ * matrix and one GEMM are faster than the convolution (wide layers on few
+ * pixels, rows that leave no 16-byte groups), that is what runs; the input
+ * gradient's long sums then go in the K slices that work gives nn_gemm_bf16.
+ * With less scratch, or none, the convolutions run.  nn_conv3_col_elems: the
+ * words that a layer has a use for, 0 where none. */
+int nn_conv3_col_elems(int ci, int co, int B, int H, int W, long long *elems);
+int nn_conv3_fwd_col(const float *x, const float *w, const float *bias, float *y, int ci, int co, int B, int H, int W,
+                     int relu, float *work, long long work_elems, float *col, long long col_elems, void *stream);
+int nn_conv3_dgrad_col(const float *dy, const float *w, float *dx, int ci, int co, int B, int H, int W, int add, float *work,
+                       long long work_elems, float *col, long long col_elems, void *stream);
+
 /* y[c][p] = act(y[c][p] + bias[c]) for c < Cout, p < P; act = ReLU if relu. */
 int nn_bias_act(float *y, const float *bias, int Cout, long long P, int relu, void *stream);
 

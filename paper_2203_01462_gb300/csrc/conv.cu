@@ -45,6 +45,8 @@
 #include <limits.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "../../include/surrogate.h"
 #include "launch.cuh"
 
@@ -962,6 +964,34 @@ void conv3(const float *in, const float *w, const float *bias, float *out, int c
     }
 }
 
+// Where the im2col matrix and one GEMM are faster: wide layers on few pixels,
+// whose convolutions are few blocks with a long serial sum each, and the gather
+// kernels, which multiply at half the GEMM's rate.  Estimates in us, fitted to
+// 180 layers (base 8 to 128, 3 x 3 to 256 x 256 pixels; us, convolution / columns):
+// input gradient 768 -> 768 7 x 7 x 2 250 / 35, 192 -> 192 32 x 32 59 / 22, 96 -> 96
+// 64 x 64 21 / 20, 24 -> 24 256 x 256 9.3 / 48; forward 512 -> 512 18 x 18 80 / 45,
+// 96 -> 96 50 x 50 x 4 80 / 61, 288 -> 96 16 x 16 x 8 33 / 39.  The convolution is
+// left only for a gain of a seventh.
+bool columns(double conv, double gemm) { return gemm < 0.87 * conv; }
+
+bool columns_fwd(int ci, int co, long long P, int W)
+{
+    if (tiled(W)) return false;
+    const double gf = 18e-9 * ci * co * P, pass = 18e-6 * ci * P;  // the products, the matrix through memory
+    return columns(std::max(15.0, 48.0 * gf), 14.0 + 20.0 * gf + pass);
+}
+
+bool columns_dgrad(int ci, int co, long long P, int W)
+{
+    const double gf = 18e-9 * ci * co * P;
+    double conv;  // of a tap, or a few, at a time: the depth is one chain
+    if (!tiled(W)) conv = std::max(0.33 * co, 28.0 * gf);
+    else if (co <= 96) conv = std::max(0.22 * co, 7.0 * gf);  // (all taps' or three taps' weights, two blocks per SM)
+    else conv = std::max(0.33 * co, 18.0 * gf * ((W + 31) / 32 * 32) / W);
+    const double pass = 36.0 * ci * P > 48e6 ? 18e-6 * ci * P : 0.0;  // the matrix stays in L2 otherwise
+    return columns(conv, 12.0 + 16.0 * gf + pass);
+}
+
 }  // namespace
 
 extern "C" {
@@ -1039,6 +1069,38 @@ int nn_conv3_wgrad(const float *dy, const float *x, float *gw, int ci, int co, i
         fdtd::launch_pdl_smem(k_conv3_wgrad<3, 2, 4>, dim3(gx, (co + 95) / 96, splits), 256, 0, st, dy, x, gw, ci, co, P, H, W, kc, work);
     if (splits > 1) fdtd::launch_pdl_smem(k_slices, slice_blocks((long long)co * N, 64), 64, 0, st, gw, work, (long long)co * N, splits);
     return status();
+}
+
+int nn_conv3_col_elems(int ci, int co, int B, int H, int W, long long *elems)
+{
+    if (!elems || !sizes_ok(ci, co, B, H, W)) return 1;
+    const long long P = (long long)B * H * W;
+    *elems = columns_fwd(ci, co, P, W) || columns_dgrad(ci, co, P, W) ? 9LL * ci * P : 0;
+    return 0;
+}
+
+int nn_conv3_fwd_col(const float *x, const float *w, const float *bias, float *y, int ci, int co, int B, int H, int W,
+                     int relu, float *work, long long work_elems, float *col, long long col_elems, void *stream)
+{
+    const long long P = (long long)B * H * W;
+    if (!col || !sizes_ok(ci, co, B, H, W) || !columns_fwd(ci, co, P, W) || col_elems < 9LL * ci * P || !bias)
+        return nn_conv3_fwd(x, w, bias, y, ci, co, B, H, W, relu, work, work_elems, stream);
+    const int K = 9 * ci, N = (int)P;
+    int rc = nn_im2col3(x, ci, B, H, W, col, stream);
+    if (!rc) rc = nn_gemm_bf16(0, 0, co, N, K, 1.0f, w, K, col, N, 0.0f, y, N, work, work_elems, stream);
+    return rc ? rc : nn_bias_act(y, bias, co, P, relu, stream);
+}
+
+int nn_conv3_dgrad_col(const float *dy, const float *w, float *dx, int ci, int co, int B, int H, int W, int add, float *work,
+                       long long work_elems, float *col, long long col_elems, void *stream)
+{
+    const long long P = (long long)B * H * W;
+    if (!col || !dx || !sizes_ok(ci, co, B, H, W) || !columns_dgrad(ci, co, P, W) || col_elems < 9LL * ci * P)
+        return nn_conv3_dgrad(dy, w, dx, ci, co, B, H, W, add, stream);
+    const int K = 9 * ci, N = (int)P;
+    int rc = nn_gemm_bf16(1, 0, K, N, co, 1.0f, w, K, dy, N, 0.0f, col, N, work, work_elems, stream);
+    if (!rc && !add) rc = nn_zero(dx, ci * P, stream);
+    return rc ? rc : nn_col2im3_add(col, ci, B, H, W, dx, stream);
 }
 
 }  // extern "C"
