@@ -181,7 +181,9 @@ typedef struct fdtd_info {
     long long launches;           /* kernels launched since create             */
     long long cell_updates;       /* cells x steps advanced since create       */
     size_t workspace_bytes;
-    long long step_blocks;        /* 2D E_z: thread blocks of one step launch  */
+    long long step_blocks;        /* 2D E_z: thread blocks of a launch of one
+                                     step (fdtd_set_steps_per_launch(1); blocked
+                                     launches have their own)                  */
     long long vector_blocks;      /* 2D E_z: of those, blocks whose tile and
                                      its one-node halo are clear of walls and
                                      CPML, which run the 16-byte vector path;
@@ -284,7 +286,8 @@ fdtd_status fdtd_set_filter_width(fdtd_ctx *ctx, double sigma);
  * they go into the FP64 accumulators: about as far from the exact sums as FP64
  * additions would be (1e-15 relative, rms).
  *
- * 3D contexts ignore the setting (see fdtd_set_wavefront). */
+ * 3D contexts ignore the setting (see fdtd_set_wavefront).  FDTD_EINVAL outside
+ * [1, 4096]: once set, the number cannot be left to the library again. */
 fdtd_status fdtd_set_steps_per_launch(fdtd_ctx *ctx, int steps);
 
 /* 3D contexts: time steps per wavefront launch of the leapfrog (Eq. 10,

@@ -308,10 +308,10 @@ struct Rt2D {
     double *G;
     PairScale ps;   // adjoint, FP32
 };
-// Halo, tile sides, warps per block, blocks along x and y, and the rounding
-// form of the Drude update (kernels_rt2d.cu, FORM).
+// Halo, tile sides, warps per block, blocks along x and y, the rounding form
+// of the Drude update (kernels_rt2d.cu, FORM), and the SMs planned for.
 struct Rt2DPlan {
-    int halo, tw, th, nw, bx, by, form;
+    int halo, tw, th, nw, bx, by, form, sms;
 };
 template <typename R>
 Rt2DPlan rt2d_plan(int nx, int ny, int sms, int steps);

@@ -778,11 +778,11 @@ int launch_rt2d(int mode, const Geo2D &g, const State2D<R> &in, const State2D<R>
                 const Pml1D<R> &py, const Rt2D<R> &w, const Rt2DPlan &p, cudaStream_t st)
 {
     if constexpr (sizeof(R) == 4) {
-        if (p.bx * p.by <= 152) {
+        if (p.bx * p.by <= p.sms) {
             launch_nb<R, 0>(mode, g, in, out, slot, px, py, w, p, st);
             return 1;
         }
-        if (p.bx * p.by > 4 * 152 && (mode == 0 || 8 * background_tiles<R>(g, p) >= 5 * p.bx * p.by)) {
+        if (p.bx * p.by > 4 * p.sms && (mode == 0 || 8 * background_tiles<R>(g, p) >= 5 * p.bx * p.by)) {
             launch_nb<R, 2>(mode, g, in, out, slot, px, py, w, p, st);
             return 1;
         }

@@ -172,7 +172,7 @@ inline Rt2DPlan rt_tile_plan(int nx, int ny, int sms, int W, int rpw, int maxw, 
             const double k = (double)waves * (fixed / H + th + H + 1);
             if (best.halo == 0 || k < cost) {
                 cost = k;
-                best = Rt2DPlan{H, tw, th, nw, bx, by, 1};
+                best = Rt2DPlan{H, tw, th, nw, bx, by, 1, sms};
             }
         }
     }
