@@ -72,6 +72,25 @@ def workload(name: str, nsteps: int | None):
 NCU_TRAFFIC_PER_STEP = {"cfg_2d_2048": 14.5e6, "cfg_3d_256": 1298.4e6}
 
 
+def roofline(w: dict, blocked: bool, achieved: float, hbm: float, peak_src: str, bytes_per_step: float) -> dict:
+    """The forward step against its bound.  achieved: GB/s on the bytes of steps
+    that each read and write the whole state.  Blocked 2D launches run several
+    steps with the state on chip (fewer launches than steps): bound by
+    instruction issue and latency, they move a fraction of those bytes, and
+    the figure is no share of a bandwidth."""
+    if w["ndim"] == 3:
+        kernel = "k_h3d + k_e3d<float,0> (forward H and E half steps; a plane wave's face corrections inside them)"
+    elif I.inplane(w):
+        kernel = "k_rt2dp (blocked forward leapfrog steps, E in plane)" if blocked else "k_hp + k_ep (forward half steps, E in plane)"
+    else:
+        kernel = "k_rt2d (blocked forward leapfrog steps)" if blocked else "k_step2d (fused forward leapfrog step)"
+    blocked = blocked and w["ndim"] == 2
+    return dict(bound="issue" if blocked else "hbm", achieved=None if blocked else achieved, peak=None if blocked else hbm,
+                unit="GB/s", frac=None if blocked else achieved / hbm, unblocked_equivalent=achieved if blocked else None,
+                traffic=NCU_TRAFFIC_PER_STEP.get(w.get("name")), traffic_unit="bytes per forward step",
+                algorithmic_bytes_per_step=bytes_per_step, kernel=kernel, peak_source=peak_src)
+
+
 def damping(k: int) -> float:
     """Artificial-damping schedule: gamma x10 decaying geometrically to x1 over 50 iterations."""
     return 10.0 ** (1.0 - min(k, 50) / 50.0)
@@ -240,7 +259,7 @@ def surrogate_measure(args) -> dict:
     rho0s = [I.zero_gap(w, 0.02 * I.rho_uniform(w, 300 + k)) for k in range(args.sur_trajectories)]
     # the training trajectories are independent: they run side by side
     pairs = collect_pairs_concurrent(w, rho0s, iters=args.sur_pairs_per_trajectory, move=0.05, damping_start=g0,
-                                     damping_iters=D, width=args.sur_trajectories, steps_per_launch=1)
+                                     damping_iters=D, width=args.sur_trajectories)
     torch.cuda.synchronize()
     collect_s = time.perf_counter() - t
     tr = Trainer(256, 256, base=24, batch=8, seed=0, lr=1e-3)
@@ -285,8 +304,8 @@ def surrogate_measure(args) -> dict:
                 wall_time_ratio_amortised=dict(designs=R, ratio=(sur_s + pre / R) / plain_s),
                 break_even_designs=(pre / (plain_s - sur_s)) if plain_s > sur_s else None,
                 pretraining=dict(pairs=len(pairs), damping_levels_in_pairs=len(levels), collect_s=collect_s,
-                                 collect="%d trajectories side by side, one solver and CUDA stream each, "
-                                 "one launch per step" % args.sur_trajectories,
+                                 collect="%d trajectories side by side, one solver and CUDA stream each"
+                                 % args.sur_trajectories,
                                  train_steps=args.sur_train_steps, train_s=train_s, final_loss=loss))
     return line
 
@@ -459,16 +478,7 @@ def main() -> None:
                     snapshot_every=w["snapshot_every"], snapshot_dtype=w.get("snapshot_dtype", "f32"),
                     parallelism="replicas" if world > 1 else "1 GPU",
                     l2="flushed (256 MB write) between timed steps"),
-        # (2D runs several steps per launch with the state on chip: the figure,
-        # on the bytes of steps that each read and write it, exceeds the copy)
-        roofline=dict(bound="hbm" if w["ndim"] == 3 else "issue", achieved=achieved, peak=hbm, unit="GB/s", frac=achieved / hbm,
-                      traffic=NCU_TRAFFIC_PER_STEP.get(w["name"]), traffic_unit="bytes per forward step",
-                      algorithmic_bytes_per_step=ab["forward"],
-                      kernel=("k_rt2dp<float,0> (blocked forward leapfrog steps, E in plane)" if I.inplane(w)
-                              else "k_rt2d<float,0> (blocked forward leapfrog steps)") if w["ndim"] == 2
-                      else "k_h3d + k_e3d<float,0> (forward H and E half steps; a plane wave's face corrections "
-                      "inside them)",
-                      peak_source=peak_src),
+        roofline=roofline(w, launches < 2 * N * args.steps, achieved, hbm, peak_src, ab["forward"]),
         phases_ms=dict(forward=statistics.median(fwd_ms), adjoint_with_recompute=statistics.median(adj_ms)),
         # every sweep the method runs: with checkpoints the adjoint phase also
         # recomputes the forward once

@@ -90,9 +90,9 @@ def collect_pairs_concurrent(w: dict, rho0_list, iters: int, move: float = 0.05,
     trajectories (one partial wave of blocks each) share the GPU.  Every
     trajectory computes exactly what collect_pairs computes (same kernels,
     same inputs); the pairs are kept in trajectory order.  steps_per_launch
-    (None: the library's default) sets the solvers' steps per launch: side
-    by side, one launch per step shares the GPU better than temporally
-    blocked launches, which each hold about a hundred SMs."""
+    (None: the library's default) sets the solvers' steps per launch.  316^2
+    FP32, ms per pair: 9.7 one after the other, 7.3 with 4 to 16 side by side;
+    with one launch per step, 16 side by side, 20."""
     pairs = pairs or Pairs()
     for b0 in range(0, len(rho0_list), width):
         group = list(rho0_list[b0:b0 + width])
