@@ -116,14 +116,14 @@ class UNet:
                   "dec1a": buf(b, 0), "dec1b": buf(b, 0), "head": buf(1, 0)}
         self.g = {k: torch.zeros_like(v) for k, v in self.a.items()}
         self.skip = {"enc1b": ("cat1", 2 * b, b), "enc2b": ("cat2", 4 * b, 2 * b), "enc3b": ("cat3", 8 * b, 4 * b)}
+        self._col_full = max(ci * k * k * B * sz[self._level(n)][0] * sz[self._level(n)][1]
+                             for n, ci, co, k in self.layers)
+        self.col = self.dcol = None  # the FP32 network's im2col matrices (_columns)
         if precision == "f32":
-            col_elems = max(ci * k * k * B * sz[self._level(n)][0] * sz[self._level(n)][1]
-                            for n, ci, co, k in self.layers)
-            self.col = torch.zeros(col_elems, **f32)
-            self.dcol = torch.zeros(col_elems, **f32)
-        else:  # the BF16 convolutions gather their operands themselves, but for layers that are faster by im2col
-            self.col = torch.zeros(max(self._col_elems(ci, co, B, *sz[self._level(n)])
-                                       for n, ci, co, k in self.layers if k == 3), **f32)
+            self._columns()
+        # the BF16 convolutions gather their operands themselves, but for layers that are faster by im2col
+        self.col_bf16 = torch.zeros(max(self._col_elems(ci, co, B, *sz[self._level(n)])
+                                        for n, ci, co, k in self.layers if k == 3), **f32)
         # split-K scratch of the GEMMs (partial products summed in a fixed
         # order): room for 16 slices of the largest weight matrix
         self.gemm_work = torch.zeros(max(1 << 20, 16 * max(co * ci * k * k for n, ci, co, k in self.layers)), **f32)
@@ -155,6 +155,14 @@ class UNet:
         return {"enc1a": 0, "enc1b": 0, "enc2a": 1, "enc2b": 1, "enc3a": 2, "enc3b": 2, "bota": 3, "botb": 3,
                 "dec3a": 2, "dec3b": 2, "dec2a": 1, "dec2b": 1, "dec1a": 0, "dec1b": 0, "head": 0}[name]
 
+    def _columns(self) -> None:
+        """Room for the largest im2col matrix and its gradient, which FP32
+        products need (also when ``precision`` is set on a BF16 network)."""
+        if self.col is None:
+            with torch.cuda.stream(self.stream):
+                self.col = torch.zeros(self._col_full, dtype=torch.float32, device=self.dev)
+                self.dcol = torch.zeros_like(self.col)
+
     @staticmethod
     def _col_elems(ci: int, co: int, B: int, H: int, W: int) -> int:
         n = C.c_longlong(0)
@@ -185,10 +193,11 @@ class UNet:
         Bhw = x[0].numel()
         if k == 3 and self.precision == "bf16":
             _ck(L.nn_conv3_fwd_col(_p(x), _p(self.w[name]), _p(self.b[name]), _p(y), ci, co, self.B, x.shape[2], x.shape[3],
-                                   int(relu), _p(self.gemm_work), self.gemm_work.numel(), _p(self.col), self.col.numel(),
-                                   st), "conv fwd")
+                                   int(relu), _p(self.gemm_work), self.gemm_work.numel(), _p(self.col_bf16),
+                                   self.col_bf16.numel(), st), "conv fwd")
             return
         if k == 3:
+            self._columns()
             _ck(L.nn_im2col3(_p(x), ci, self.B, x.shape[2], x.shape[3], _p(self.col), st), "im2col")
             src = self.col
         else:
@@ -206,10 +215,11 @@ class UNet:
                                  _p(self.gemm_work), self.gemm_work.numel(), st), "conv wgrad")
             if dx is not None:
                 _ck(L.nn_conv3_dgrad_col(_p(dy), _p(self.w[name]), _p(dx), ci, co, self.B, x.shape[2], x.shape[3], 0,
-                                         _p(self.gemm_work), self.gemm_work.numel(), _p(self.col), self.col.numel(),
-                                         st), "conv dgrad")
+                                         _p(self.gemm_work), self.gemm_work.numel(), _p(self.col_bf16),
+                                         self.col_bf16.numel(), st), "conv dgrad")
             return
         if k == 3:
+            self._columns()
             _ck(L.nn_im2col3(_p(x), ci, self.B, x.shape[2], x.shape[3], _p(self.col), st), "im2col")
             src = self.col
         else:
