@@ -53,7 +53,7 @@ struct Shape {
     static constexpr int VX = sizeof(R) == 4 ? 2 : 1;
     static constexpr int RPW = sizeof(R) == 4 ? 2 : 1;
     static constexpr int W = 32 * VX;   // region width
-    static constexpr int MAXW = sizeof(R) == 4 ? 16 : 24;  // warps per block (FP32: 128 registers a thread)
+    static constexpr int MAXW = sizeof(R) == 4 ? 16 : 24;  // warps per block (FP32: 128 registers a thread; the adjoint spills 88 to 128 B)
 };
 
 // Shared memory of one block (in words of R unless noted), in this order:
@@ -769,7 +769,7 @@ int background_tiles(const Geo2D &g, const Rt2DPlan &p)
 // stores then overlap the other's steps.  us per forward step, one and two
 // blocks per SM: 700^2 (3.2 waves) 3.13 / 3.15, 850^2 (4.8) 3.87 / 3.75, 1400^2
 // 8.0 / 6.9, 2048^2 17.8 / 13.2, 1500^2 nearly all design box 13.0 / 11.3.  The
-// adjoint, which spills 1.9 kB outside the background, takes it where five
+// adjoint, which spills 2 kB outside the background, takes it where five
 // eighths of the tiles are background: 2048^2 with a 1024^2 design box (66 %)
 // 22.3 / 19.6, 2200 x 1000 with 300^2 (80 %) 9.3 / 8.5, but 1200^2 with 600^2
 // (58 %) 8.3 / 8.9 and 1500^2 with 1400^2 (5 %) 20.1 / 22.5.
