@@ -429,13 +429,18 @@ __global__ void __launch_bounds__(32 * Shape<R>::MAXW, 1)
     }
 }
 
+// (Blocks of two warps: with 164 registers a thread three of four fit on an SM,
+// and a design box of one to two waves ended with a few blocks alone; 1 % of an
+// evaluation of small boxes.)
+constexpr int SENS_TPB = 64;
+
 // Sensitivities of `count` adjoint steps of the pitched design edges (both
 // components): step t went from adjoint E ae[t - 1] (t = 0: eprev) to ae[t],
 // with the forward E fe[-t] of its source time.  jsens is the adjoint J
 // before the first step and is advanced; eprev receives the last E.  A thread
 // owns 16 bytes of adjacent edges and keeps U steps' loads in flight.
 template <typename R>
-__global__ void __launch_bounds__(128) k_rt2dp_sens(int slot, long long M0, long long M1, const R *__restrict__ coef0,
+__global__ void __launch_bounds__(SENS_TPB) k_rt2dp_sens(int slot, long long M0, long long M1, const R *__restrict__ coef0,
                                                     const R *__restrict__ coef1, long long step,
                                                     const R *__restrict__ ae, const R *__restrict__ fe, int count,
                                                     R *j0, R *j1, R *e0, R *e1, double *G0, double *G1, PairScale ps)
@@ -443,8 +448,8 @@ __global__ void __launch_bounds__(128) k_rt2dp_sens(int slot, long long M0, long
     constexpr int V = 16 / sizeof(R), U = 8;
     const Coef<R> &c = coef_at<R>(slot);
     // threads past the end work on the last edges and store nothing
-    const long long id = min((blockIdx.x * 128LL + threadIdx.x) * V, M0 + M1 - V);
-    const bool inside = (blockIdx.x * 128LL + threadIdx.x) * V < M0 + M1;
+    const long long id = min((blockIdx.x * (long long)SENS_TPB + threadIdx.x) * V, M0 + M1 - V);
+    const bool inside = (blockIdx.x * (long long)SENS_TPB + threadIdx.x) * V < M0 + M1;
     const bool second = id >= M0;
     const long long q = second ? id - M0 : id, M = second ? M1 : M0;
     const R *coef = (second ? coef1 : coef0) + q;
@@ -612,7 +617,7 @@ int launch_rt2dp_sens(const GeoP &g, int slot, const R *const coef[2], long long
 {
     constexpr int V = 16 / sizeof(R);
     const long long n = g.Mdi[0] + g.Mdi[1];
-    launch_pdl(k_rt2dp_sens<R>, dim3((unsigned)((n + 128 * V - 1) / (128 * V))), dim3(128), st, slot, (long long)g.Mdi[0],
+    launch_pdl(k_rt2dp_sens<R>, dim3((unsigned)((n + SENS_TPB * V - 1) / (SENS_TPB * V))), dim3(SENS_TPB), st, slot, (long long)g.Mdi[0],
                (long long)g.Mdi[1], coef[0], coef[1], step, ae, fe, count, jsens[0], jsens[1], eprev[0], eprev[1], G[0], G[1],
                ps);
     return 1;
